@@ -1312,9 +1312,10 @@ __device__ void jo_count_in(const DevScene& sc, const Job& J, const float* P, co
     const int npx = nu * nv;
     const float rr = __fmul_rn(J.m.vol_r, J.m.vol_r);
     for (;;) {
-        if (stop && *reinterpret_cast<const volatile int*>(stop) >= NT / 32) break;
-        int c = 0;
-        if (lane == 0) c = atomicAdd(counter, 1);
+        // one lane looks whether to stop and takes the chunk, so that the warp
+        // leaves the loop as one whatever the other warps do meanwhile
+        int c = INT_MAX / kJoChunk;
+        if (lane == 0 && !(stop && *reinterpret_cast<const volatile int*>(stop) >= NT / 32)) c = atomicAdd(counter, 1);
         const int k0 = __shfl_sync(0xffffffffu, c, 0) * kJoChunk;
         if (k0 >= npx) break;
         const int k1 = min(k0 + kJoChunk, npx);
