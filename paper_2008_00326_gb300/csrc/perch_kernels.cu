@@ -586,7 +586,6 @@ __device__ __forceinline__ void zmin(uint32_t* zbuf, int idx, unsigned d, int tr
 // ---- resolve queue and per-warp cell groups -------------------------------
 
 constexpr int kWarpQueue = 64;    // kept rendered points queued per warp (a ring)
-constexpr int kGroups = 1;        // distinct query cells looked up together per warp
 
 // A group of G queries shares a 27-cell candidate list; k = floor(32 / G)
 // lanes test each query's candidates.  Lane l serves query floor(l / k),
@@ -606,13 +605,14 @@ struct __align__(16) KeptPoint {  // a rendered point of R \ C waiting for its r
 
 // Per-warp scratch of the radius search (shared memory).
 struct __align__(16) WarpProbe {
-    int2 runs[kGroups][27];       // per group: non-empty runs as (start - first pair index, end pair index)
-    int total[kGroups];           // per group: candidates in its 27 cells
-    unsigned mask[kGroups];       // per group: lanes whose query lies in the group's cell
-    unsigned char qlist[kGroups][32];  // per group: the lanes of its queries, in lane order
-    float4 q[32];                 // query of each lane
-    unsigned long long best[32];  // nearest-neighbour key of each lane's query
-    float4 stage[64];             // a chunk of the group's candidates, shared by its queries
+    int2 runs[27];                // hash: non-empty cells as (start - first candidate, end candidate);
+                                  // dense index: runs[r].x of the non-empty rows
+    int total;                    // hash: candidates of the group's 27 cells
+    unsigned char qlist[32];      // hash: the lanes of the group's queries, in lane order
+    float4 q[32];                 // query of each lane (dense index: -x, -x, -y, -y)
+    unsigned long long best[32];  // hash: nearest-neighbour key of each lane's query
+    float4 stage[64];             // hash: a chunk of the group's candidates, shared by its queries;
+                                  // dense index: .xy = -z, -z of each lane's query
 };
 
 // Per-warp scratch: the radius search and the rasteriser's triangle stage
@@ -624,78 +624,43 @@ static_assert(sizeof(TriStage) == 64, "staged triangles are 64 bytes");
 static_assert(kWarpScratch % 16 == 0, "per-warp scratch keeps 16-byte alignment");
 static_assert(sizeof(WarpProbe) % 16 == 0, "per-warp scratch keeps 16-byte alignment");
 
-// Warp-cooperative lookup of the 27-cell neighbourhoods of up to kGroups
-// query cells at once.  With the dense cell index, lane j < 9 reads the two
-// bounds of one row's three cells (they are contiguous); otherwise lane
-// j < 27 probes the hash table for neighbour j, issuing all first-slot loads
-// before resolving any (the table lives in L2, so the loads overlap).  Group
-// g's non-empty runs are stored in order with a running candidate count so
-// that candidate i of the group is point runs[r].x + i for the first run r
-// with i < runs[r].y.
-__device__ __forceinline__ void lookup_cells(const DevScene& sc, const int* gx, const int* gy,
-                                             const int* gz, int ng, WarpProbe& W, int lane, int* nruns)
+// Warp-cooperative lookup of the 27 cells around cell (gx, gy, gz) in the voxel
+// hash (an observation whose cell box is too large for the dense index): lane
+// j < 27 probes the table for neighbour j (the table lives in L2, so the loads
+// overlap).  The non-empty runs are stored in order with a running candidate
+// count, so that candidate i is point runs[r].x + i for the first run r with
+// i < runs[r].y.  Returns the number of runs.
+__device__ __forceinline__ int lookup_hash(const DevScene& sc, int gx, int gy, int gz, WarpProbe& W, int lane)
 {
-    const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) {
-        if (g >= ng) break;
-        uint32_t start = 0, cnt = 0;
-        if (sc.cell_start) {
-            // dense index: lane j < 9 takes row (y + j % 3 - 1, z + j / 3 - 1),
-            // whose cells x-1..x+1 are one run of the cell-sorted points
-            if (lane < 9) {
-                const int ry = gy[g] + lane % 3 - 1 - sc.near_lo[1], rz = gz[g] + lane / 3 - 1 - sc.near_lo[2];
-                const int x0 = max(gx[g] - 1 - sc.near_lo[0], 0), x1 = min(gx[g] + 1 - sc.near_lo[0], sc.near_n[0] - 1);
-                if (ry >= 0 && ry < sc.near_n[1] && rz >= 0 && rz < sc.near_n[2] && x0 <= x1) {
-                    const long long row = ((long long)rz * sc.near_n[1] + ry) * sc.near_n[0];
-                    start = __ldg(&sc.cell_start[row + x0]);
-                    cnt = __ldg(&sc.cell_start[row + x1 + 1]) - start;
-                }
+    uint32_t start = 0, cnt = 0;
+    if (lane < 27) {
+        const unsigned long long key = cell_key(gx + lane % 3 - 1, gy + (lane / 3) % 3 - 1, gz + lane / 9 - 1);
+        uint32_t slot = hash_slot(key, sc.table_mask);
+        for (uint32_t probe = 0; probe <= sc.table_mask; ++probe) {
+            const uint4 x = __ldg(&sc.table[slot]);
+            unsigned long long k = (unsigned long long)x.x | ((unsigned long long)x.y << 32);
+            if (k == key) {
+                start = x.z;
+                cnt = x.w;
+                break;
             }
-        } else if (lane < 27) {
-            // voxel hash (a cell box too large for the dense index): lane j
-            // probes the table for neighbour j
-            const unsigned long long key = cell_key(gx[g] + dx, gy[g] + dy, gz[g] + dz);
-            uint32_t slot = hash_slot(key, sc.table_mask);
-            for (uint32_t probe = 0; probe <= sc.table_mask; ++probe) {
-                const uint4 x = __ldg(&sc.table[slot]);
-                unsigned long long k = (unsigned long long)x.x | ((unsigned long long)x.y << 32);
-                if (k == key) {
-                    start = x.z;
-                    cnt = x.w;
-                    break;
-                }
-                if (k == kEmptyKey) break;
-                slot = (slot + 1) & sc.table_mask;
-            }
+            if (k == kEmptyKey) break;
+            slot = (slot + 1) & sc.table_mask;
         }
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const unsigned nonempty = __ballot_sync(0xffffffffu, cnt != 0);
-        if (cnt != 0)
-            W.runs[g][__popc(nonempty & ((1u << lane) - 1u))] =
-                make_int2((int)start - (int)(incl - cnt), (int)incl);
-        if (lane == 31) W.total[g] = (int)incl;
-        nruns[g] = __popc(nonempty);
     }
+    uint32_t incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const unsigned nonempty = __ballot_sync(0xffffffffu, cnt != 0);
+    if (cnt != 0)
+        W.runs[__popc(nonempty & ((1u << lane) - 1u))] = make_int2((int)start - (int)(incl - cnt), (int)incl);
+    if (lane == 31) W.total = (int)incl;
+    return __popc(nonempty);
 }
 
-// Radius search for up to 32 queued points (one per lane; `valid` marks the
-// lanes holding one).  Lanes whose points fall in the same hash cell form a
-// group (__match_any_sync); each group's 27-cell neighbourhood is looked up
-// once, cooperatively.  The group's candidates are then staged in shared
-// memory 64 at a time (two coalesced loads per lane, each candidate loaded
-// once however many of the group's queries test it) and tested by all 32
-// lanes: floor(32 / G) lanes per query (G = the group's queries) split each
-// chunk, each keeps its minimum (d2 bits, pixel) in a register and folds it
-// into the query's result with one shared-memory atomicMin.  Returns the
-// lane's own result: the nearest observed point within delta (smallest FP32
-// squared distance, ties to the lowest pixel index) or kEmptyKey.  All 32
-// lanes must call it.
 // Admissible band of the observed-side keys (jo_mode 1: for every observed
 // point of the band, the key (d2 bits << 32 | rendered pixel) of its nearest
 // rendered point within delta, kEmptyKey if none).
@@ -761,16 +726,22 @@ __device__ __forceinline__ void stage_chunk(const DevScene& sc, WarpProbe& W, in
     if (cj < T && PERCH_CHECKED((unsigned)pj < (unsigned)sc.n_pts, err)) W.stage[lane + 32] = __ldg(&sc.pts[pj]);
 }
 
+// Radius search of up to 32 points through the voxel hash.  Lanes whose points
+// fall in the same cell form a group; its 27-cell neighbourhood is looked up
+// once, its candidates are staged in shared memory 64 at a time and tested by
+// all 32 lanes: floor(32 / G) lanes per query (G = the group's queries) split
+// each chunk, each keeps its minimum (d2 bits, pixel) in a register and folds
+// it into the query's result with one shared-memory atomicMin.
 template <bool MARK>
-__device__ unsigned long long probe_batch(const DevScene& sc, bool valid, float qx, float qy,
-                                          float qz, uint32_t qpix, WarpProbe& W, int lane, const MarkBand& mb)
+__device__ __noinline__ unsigned long long probe_hash(const DevScene& sc, bool valid, float4 query, WarpProbe& W,
+                                                      int lane, const MarkBand& mb)
 {
     int cx = 0, cy = 0, cz = 0;
     unsigned long long key = kEmptyKey;
     if (valid) {
-        cx = cell_coord(qx, sc.inv_cell);
-        cy = cell_coord(qy, sc.inv_cell);
-        cz = cell_coord(qz, sc.inv_cell);
+        cx = cell_coord(query.x, sc.inv_cell);
+        cy = cell_coord(query.y, sc.inv_cell);
+        cz = cell_coord(query.z, sc.inv_cell);
         if (sc.near_bits) {
             // no observed point in the 27 cells: nothing to look up
             const long long b = near_index(sc, cx, cy, cz);
@@ -778,62 +749,247 @@ __device__ unsigned long long probe_batch(const DevScene& sc, bool valid, float 
         }
         if (valid) key = cell_key(cx, cy, cz);
     }
-    W.q[lane] = make_float4(qx, qy, qz, __uint_as_float(qpix));
+    W.q[lane] = query;
     W.best[lane] = kEmptyKey;
     const unsigned grp = __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(grp) - 1;
-    const unsigned leaders = __ballot_sync(0xffffffffu, valid && lane == leader);
-    const int my_g = __popc(leaders & ((1u << leader) - 1u));
     const int my_pos = __popc(grp & ((1u << lane) - 1u));
-    unsigned rest = leaders;
-    for (int g0 = 0; rest != 0; g0 += kGroups) {
-        int gx[kGroups], gy[kGroups], gz[kGroups];
-        int ng = 0;
-#pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-            gx[g] = gy[g] = gz[g] = 0;
-            if (rest != 0) {
-                const int L = __ffs(rest) - 1;
-                rest &= rest - 1;
-                gx[g] = __shfl_sync(0xffffffffu, cx, L);
-                gy[g] = __shfl_sync(0xffffffffu, cy, L);
-                gz[g] = __shfl_sync(0xffffffffu, cz, L);
-                const unsigned m = __shfl_sync(0xffffffffu, grp, L);
-                if (lane == 0) W.mask[g] = m;
-                ng = g + 1;
-            }
-        }
-        if (valid && my_g >= g0 && my_g < g0 + kGroups) W.qlist[my_g - g0][my_pos] = (unsigned char)lane;
-        int nruns[kGroups];
-        lookup_cells(sc, gx, gy, gz, ng, W, lane, nruns);
+    for (unsigned rest = __ballot_sync(0xffffffffu, valid && lane == leader); rest != 0; rest &= rest - 1) {
+        const int L = __ffs(rest) - 1;
+        if (valid && leader == L) W.qlist[my_pos] = (unsigned char)lane;
+        const int nruns = lookup_hash(sc, __shfl_sync(0xffffffffu, cx, L), __shfl_sync(0xffffffffu, cy, L),
+                                      __shfl_sync(0xffffffffu, cz, L), W, lane);
+        const int G = __popc(__shfl_sync(0xffffffffu, grp, L));
         __syncwarp();
-        for (int g = 0; g < ng; ++g) {
-            const int T = W.total[g];
-            if (T == 0) continue;
-            // k = floor(32 / G) lanes per query; lane j of a query takes
-            // candidates j, j + k, ... of each staged chunk and keeps its
-            // minimum in a register
-            const int G = __popc(W.mask[g]);
-            const int k = c_lanes_per_query[G];
-            const int qj = (lane * (int)c_lane_div[k]) >> 10;
-            const bool active = lane < G * k;
-            const int ql = active ? W.qlist[g][qj] : 0;
-            const float4 q = W.q[ql];
-            unsigned long long local = kEmptyKey;
-            const int2 run = lane < nruns[g] ? W.runs[g][lane] : make_int2(0, INT_MAX);
-            for (int c0 = 0; c0 < T; c0 += 64) {
-                stage_chunk(sc, W, run, c0, T, lane, mb.err);
-                __syncwarp();
-                const int n = min(64, T - c0);
-                if (active)
-                    local = scan_staged<MARK>(sc, q, W.stage, n, lane - qj * k, k, mb, local);
-                __syncwarp();
-            }
-            if (active && local != kEmptyKey) atomicMin(&W.best[ql], local);
+        const int T = W.total;
+        // k = floor(32 / G) lanes per query; lane j of a query takes
+        // candidates j, j + k, ... of each staged chunk and keeps its
+        // minimum in a register
+        const int k = c_lanes_per_query[G];
+        const int qj = (lane * (int)c_lane_div[k]) >> 10;
+        const bool active = lane < G * k;
+        const int ql = active ? W.qlist[qj] : 0;
+        const float4 q = W.q[ql];
+        unsigned long long local = kEmptyKey;
+        const int2 run = lane < nruns ? W.runs[lane] : make_int2(0, INT_MAX);
+        for (int c0 = 0; c0 < T; c0 += 64) {
+            stage_chunk(sc, W, run, c0, T, lane, mb.err);
+            __syncwarp();
+            const int n = min(64, T - c0);
+            if (active) local = scan_staged<MARK>(sc, q, W.stage, n, lane - qj * k, k, mb, local);
+            __syncwarp();
         }
+        if (active && local != kEmptyKey) atomicMin(&W.best[ql], local);
         __syncwarp();
     }
     return W.best[lane];
+}
+
+// Packed binary32 pairs, each half rounded to nearest like the scalar operation.
+// A square is a fused multiply-add of the pair (-0, -0), which changes no bit of
+// the product.  The pair is read from constant memory: a packed multiplication,
+// or an addend the assembler can see through, is contracted with the addition
+// that follows it (.rn and -fmad=false notwithstanding: measured, 22 % of the
+// sums then differ in their last bit).
+__constant__ unsigned long long c_negzero2 = 0x8000000080000000ull;
+
+__device__ __forceinline__ unsigned long long pack2(float a, float b)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ unsigned long long square2(unsigned long long a)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(a), "l"(c_negzero2));
+    return r;
+}
+
+// Bits of the squared distances of a query (negated, each coordinate twice: the
+// differences only change sign) to two candidates, by packed binary32 operations
+// that round each half as the scalar ones do.  The values are non-negative, so
+// the bits order like them; a NaN compares above every radius.
+__device__ __forceinline__ uint2 dist2_pair(ulonglong2 qxy, unsigned long long qz, unsigned long long x,
+                                            unsigned long long y, unsigned long long z)
+{
+    const unsigned long long ex = add2(x, qxy.x), ey = add2(y, qxy.y), ez = add2(z, qz);
+    const unsigned long long d = add2(add2(square2(ex), square2(ey)), square2(ez));
+    return make_uint2((unsigned)d, (unsigned)(d >> 32));
+}
+
+// jo_mode 1: fold the pair (query of rendered pixel qpix, observed point of pixel
+// pw, squared distance d2) into the observed point's key if the two lie within
+// delta of each other and the point in the admissible band.
+__device__ __forceinline__ void mark_pair(const MarkBand& mb, unsigned d2, unsigned d2max, uint32_t qpix, uint32_t pw)
+{
+    if (d2 > d2max) return;
+    const int pu = (int)(pw & 0xFFFFu), pv = (int)(pw >> 16);
+    if (pu >= mb.u0 && pu < mb.u1 && pv >= mb.v0 && pv < mb.v1)
+        atomicMin(reinterpret_cast<unsigned long long*>(mb.marks) + (pv - mb.v0) * mb.vw + (pu - mb.u0),
+                  ((unsigned long long)d2 << 32) | qpix);
+}
+
+// 32 candidates c .. c + 31 of a group of T (c uniform; lane l takes c + l), one
+// per lane.  Lane j < 9 holds row j of the group: cnt points, the first of them
+// the group's candidate off.  base[r] is the point index of the r-th non-empty
+// row's candidate 0; begun counts the rows begun before c (advanced).
+__device__ __forceinline__ float4 group_candidate(const DevScene& sc, const int2* base, int off, int cnt, int c, int T,
+                                                  int lane, int& begun, int* err)
+{
+    const float far = 1.0e30f;                            // beyond every radius: d2 = inf
+    float4 p = make_float4(far, far, far, 0.0f);
+    const unsigned rel = (unsigned)(off - c);
+    const unsigned starts = __reduce_or_sync(0xffffffffu, cnt != 0 && rel < 32u ? 1u << rel : 0u);
+    if (c + lane < T) {
+        // the candidate lies in the last row begun at or before it
+        const int i = base[begun + __popc(starts & (0xffffffffu >> (31 - lane))) - 1].x + c + lane;
+        if (PERCH_CHECKED((unsigned)i < (unsigned)sc.n_pts, err)) p = __ldg(&sc.pts[i]);
+    }
+    begun += __popc(starts);
+    return p;
+}
+
+// Radius search of up to 32 points through the dense cell index.  Lanes whose
+// points fall in the same cell form a group.  The group's candidates -- nine
+// rows of three cells, each row one run of the cell-sorted points -- are held
+// two or four per lane in registers, loaded once by coalesced reads; every
+// query of the group is then broadcast to them, and the warp's minimum of the
+// squared distances and of the pixels that attain it is the query's nearest
+// point (two warp-wide integer minima).  The cell box has a border of empty
+// cells, so rows that run over its faces only wrap into empty cells or into
+// further observed points, which cannot change a nearest neighbour within
+// delta; only the ends of the whole index are clamped.  NEAR: the caller has
+// tested the near-cell bits.
+//
+// Bound by instruction issue.  A group costs about 70 instructions, a query
+// about 20 per 64 candidates (30 per 128), against the 16 to 230 candidates of
+// a mean query on the tabletop and 6-DoF scenes.  Staging the candidates in
+// shared memory and splitting the lanes over the group's queries cost about
+// twice that: three 640x480 objects x 29,584 poses 45.2 -> 42.0 ms, five 6-DoF
+// objects x 4,096 poses 27.9 -> 22.8 ms, their refinement 52.3 -> 42.7 ms.
+template <bool MARK, bool NEAR>
+__device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bool valid, float4 query, WarpProbe& W,
+                                                          int lane, const MarkBand& mb)
+{
+    const int nx = sc.near_n[0], nxy = nx * sc.near_n[1], ncell = nxy * sc.near_n[2];
+    int cell = -1;
+    if (valid) {
+        const int ix = cell_coord(query.x, sc.inv_cell) - sc.near_lo[0];
+        const int iy = cell_coord(query.y, sc.inv_cell) - sc.near_lo[1];
+        const int iz = cell_coord(query.z, sc.inv_cell) - sc.near_lo[2];
+        if ((unsigned)ix < (unsigned)nx && (unsigned)iy < (unsigned)sc.near_n[1] && (unsigned)iz < (unsigned)sc.near_n[2]) {
+            const int c = iz * nxy + iy * nx + ix;
+            if (NEAR || ((__ldg(&sc.near_bits[c >> 5]) >> (c & 31)) & 1u)) cell = c;
+        }
+    }
+    W.q[lane] = make_float4(-query.x, -query.x, -query.y, -query.y);
+    W.stage[lane] = make_float4(-query.z, -query.z, query.w, 0.0f);
+    const unsigned grp = __match_any_sync(0xffffffffu, cell);
+    const unsigned d2max = __float_as_uint(sc.delta2);
+    // lane j < 9: from a cell to the first of the three cells of its row j
+    const int row_off = (lane % 3 - 1) * nx + (lane / 3 - 1) * nxy - 1;
+    unsigned bd = 0xFFFFFFFFu, bp = 0xFFFFFFFFu;          // the lane's own nearest point
+    __syncwarp();
+    for (unsigned rest = __ballot_sync(0xffffffffu, cell >= 0 && (grp & ((1u << lane) - 1u)) == 0u); rest != 0;
+         rest &= rest - 1) {
+        const int L = __ffs(rest) - 1;
+        const int c = __shfl_sync(0xffffffffu, cell, L);
+        const unsigned members = __shfl_sync(0xffffffffu, grp, L);
+        int s0 = 0, cnt = 0;
+        if (lane < 9) {
+            s0 = (int)__ldg(&sc.cell_start[min(max(c + row_off, 0), ncell)]);
+            cnt = (int)__ldg(&sc.cell_start[min(max(c + row_off + 3, 0), ncell)]) - s0;
+        }
+        int off = cnt;                                    // the row's first candidate
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, off, o);
+            if (lane >= o) off += t;
+        }
+        const int T = __shfl_sync(0xffffffffu, off, 8);
+        off -= cnt;
+        const unsigned nonempty = __ballot_sync(0xffffffffu, cnt != 0);
+        if (cnt != 0) W.runs[__popc(nonempty & ((1u << lane) - 1u))].x = s0 - off;
+        __syncwarp();
+        int begun = 0;
+        for (int c0 = 0; c0 < T; c0 += 128) {
+            const float4 ca = group_candidate(sc, W.runs, off, cnt, c0, T, lane, begun, mb.err);
+            const float4 cb = group_candidate(sc, W.runs, off, cnt, c0 + 32, T, lane, begun, mb.err);
+            const unsigned long long x0 = pack2(ca.x, cb.x), y0 = pack2(ca.y, cb.y), z0 = pack2(ca.z, cb.z);
+            const unsigned pa = __float_as_uint(ca.w), pb = __float_as_uint(cb.w);
+            if (T - c0 <= 64) {
+                for (unsigned m = members; m != 0; m &= m - 1) {
+                    const int i = __ffs(m) - 1;
+                    const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&W.q[i]);
+                    const unsigned long long qz = *reinterpret_cast<const unsigned long long*>(&W.stage[i]);
+                    const uint2 d = dist2_pair(qa, qz, x0, y0, z0);
+                    if (MARK) {
+                        const uint32_t qp = __float_as_uint(W.stage[i].z);
+                        mark_pair(mb, d.x, d2max, qp, pa);
+                        mark_pair(mb, d.y, d2max, qp, pb);
+                    }
+                    const unsigned dm = __reduce_min_sync(0xffffffffu, min(d.x, d.y));
+                    if (dm > d2max) continue;
+                    const unsigned pm = __reduce_min_sync(
+                        0xffffffffu, min(d.x == dm ? pa : 0xFFFFFFFFu, d.y == dm ? pb : 0xFFFFFFFFu));
+                    if (lane == i && (dm < bd || (dm == bd && pm < bp))) {
+                        bd = dm;
+                        bp = pm;
+                    }
+                }
+            } else {
+                const float4 cc = group_candidate(sc, W.runs, off, cnt, c0 + 64, T, lane, begun, mb.err);
+                const float4 cd = group_candidate(sc, W.runs, off, cnt, c0 + 96, T, lane, begun, mb.err);
+                const unsigned long long x1 = pack2(cc.x, cd.x), y1 = pack2(cc.y, cd.y), z1 = pack2(cc.z, cd.z);
+                const unsigned pc = __float_as_uint(cc.w), pd = __float_as_uint(cd.w);
+                for (unsigned m = members; m != 0; m &= m - 1) {
+                    const int i = __ffs(m) - 1;
+                    const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&W.q[i]);
+                    const unsigned long long qz = *reinterpret_cast<const unsigned long long*>(&W.stage[i]);
+                    const uint2 d = dist2_pair(qa, qz, x0, y0, z0), e = dist2_pair(qa, qz, x1, y1, z1);
+                    if (MARK) {
+                        const uint32_t qp = __float_as_uint(W.stage[i].z);
+                        mark_pair(mb, d.x, d2max, qp, pa);
+                        mark_pair(mb, d.y, d2max, qp, pb);
+                        mark_pair(mb, e.x, d2max, qp, pc);
+                        mark_pair(mb, e.y, d2max, qp, pd);
+                    }
+                    const unsigned dm = __reduce_min_sync(0xffffffffu, min(min(d.x, d.y), min(e.x, e.y)));
+                    if (dm > d2max) continue;
+                    const unsigned pm = __reduce_min_sync(
+                        0xffffffffu, min(min(d.x == dm ? pa : 0xFFFFFFFFu, d.y == dm ? pb : 0xFFFFFFFFu),
+                                         min(e.x == dm ? pc : 0xFFFFFFFFu, e.y == dm ? pd : 0xFFFFFFFFu)));
+                    if (lane == i && (dm < bd || (dm == bd && pm < bp))) {
+                        bd = dm;
+                        bp = pm;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
+    return ((unsigned long long)bd << 32) | bp;
+}
+
+// Radius search for up to 32 queued points (one per lane; `valid` marks the
+// lanes holding one).  Returns the lane's own result: the nearest observed
+// point within delta (smallest FP32 squared distance, ties to the lowest pixel)
+// as (d2 bits << 32 | pixel), or kEmptyKey.  All 32 lanes must call it.
+template <bool MARK, bool NEAR>
+__device__ __forceinline__ unsigned long long probe_batch(const DevScene& sc, bool valid, float qx, float qy, float qz,
+                                                          uint32_t qpix, WarpProbe& W, int lane, const MarkBand& mb)
+{
+    const float4 q = make_float4(qx, qy, qz, __uint_as_float(qpix));
+    return sc.cell_start ? probe_dense<MARK, NEAR>(sc, valid, q, W, lane, mb) : probe_hash<MARK>(sc, valid, q, W, lane, mb);
 }
 
 // Conservative pixel box of an object-frame box [lo,hi] at pose P (2 px
@@ -1485,7 +1641,7 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
                     wq_head = (wq_head + nb) % kWarpQueue;
                     wq_count -= nb;
                     const uint32_t qpix = (EQ3 && valid) ? kq.pix : 0u;
-                    const unsigned long long nn = probe_batch<EQ3>(sc, valid, kq.x, kq.y, kq.z, qpix, WP, lane, mband);
+                    const unsigned long long nn = probe_batch<EQ3, true>(sc, valid, kq.x, kq.y, kq.z, qpix, WP, lane, mband);
                     if (valid) {
                         bool explained = nn != kEmptyKey;
                         const int pnn = (int)(uint32_t)nn;
@@ -1792,7 +1948,7 @@ __device__ int claim_vslot(unsigned* mask, int nslots)
 // fit an SM when the block's shared memory allows (the default launch shape),
 // which hides latency better than three blocks of 80 registers.
 template <int NT, int MODE, bool BINS>
-__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 1024 / NT) k_score(ScoreArgs a)
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 1024 / NT) k_score(const __grid_constant__ ScoreArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float s_pose[12];
@@ -2252,7 +2408,7 @@ __host__ __device__ inline size_t gicp_probe_offset(int zcap_words)
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) k_gicp(GicpArgs a)
+__global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ GicpArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float s_pose[12], s_Rf[9], s_tf[3];
@@ -2330,7 +2486,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(GicpArgs a)
                 const float3 r0 = rotate_rn(s_Rf, 3, A.x, A.y, A.z);
                 const float3 p = make_float3(__fadd_rn(r0.x, s_tf[0]), __fadd_rn(r0.y, s_tf[1]),
                                              __fadd_rn(r0.z, s_tf[2]));
-                const unsigned long long nn = probe_batch<false>(sc, valid, p.x, p.y, p.z, 0u, WP, lane, nomark);
+                const unsigned long long nn = probe_batch<false, false>(sc, valid, p.x, p.y, p.z, 0u, WP, lane, nomark);
                 bool ok = valid && nn != kEmptyKey;
                 float terms[kGicpTerms];
                 if (ok) {
