@@ -710,6 +710,9 @@ perch_status perch_set_observation(perch_ctx* c, const uint16_t* depth, const ui
     if (!e && labels) e = cudaMemcpyAsync(s.labels, labels, npx * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
     perch::DevScene& d = s.ds;
     d.W = W; d.H = H; d.fx = fx; d.fy = fy; d.cx = cx; d.cy = cy;
+    const bool fast = fx > 0x1p-60f && fx < 0x1p60f && fy > 0x1p-60f && fy < 0x1p60f;
+    d.rfx = fast ? 1.0f / fx : 0.0f;
+    d.rfy = 1.0f / fy;
     d.delta = p.delta_m;
     d.delta2 = p.delta_m * p.delta_m;
     d.cell = cell;
@@ -717,7 +720,7 @@ perch_status perch_set_observation(perch_ctx* c, const uint16_t* depth, const ui
     d.tau_c = p.tau_c;
     d.z_near = p.z_near_m;
     d.color_check = p.color_check;
-    d.stride = p.stride;
+    d.stride = std::min(p.stride, std::max(W, H));   // any larger stride keeps pixel (0, 0) alone too
     d.occ_margin = p.occ_margin_units;
     d.jo_mode = p.jo_mode;
     d.depth = (const uint16_t*)s.depth;

@@ -16,6 +16,7 @@ constexpr double kMaxCellCoord = 1.0e5;        // |coordinate / cell| bound for 
 struct DevScene {
     int W, H;
     float fx, fy, cx, cy;
+    float rfx, rfy;           // fl(1 / fx), fl(1 / fy); rfx = 0: out of the fast division's range
     float delta, delta2, cell, inv_cell, tau_c, z_near;   // inv_cell = fl(1 / cell)
     int color_check, stride, occ_margin;
     int jo_mode;              // 0: NN marks (Sec. IV-A kernel); 1: Eq. 3 with the Eq. 2 test
@@ -79,6 +80,9 @@ struct ScoreArgs {
     long long n;              // hypotheses (= job.n)
     int zcap_words;           // z-buffer capacity in 32-bit words
     int mark_words;           // marks bitset capacity in 32-bit words
+    // byte offsets in the block's shared memory (set by the launch): the marks,
+    // the warps' kept-point queues, their scratch; the z-buffer is at 0
+    unsigned marks_off, kept_off, probe_off;
     unsigned long long* dump; // debug: W*H 64-bit keys, or nullptr
     int* err;                 // device error word (bit flags)
     unsigned* next;           // hypothesis counter, zeroed before the launch

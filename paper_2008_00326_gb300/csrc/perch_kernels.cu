@@ -62,10 +62,18 @@ __device__ __forceinline__ float3 srgb8_to_lab(uint32_t r8, uint32_t g8, uint32_
     return make_float3(116.0f * fy - 16.0f, 500.0f * (fx - fy), 200.0f * (fy - fz));
 }
 
+// Hue angle in [0, 360) degrees, 0 on the neutral axis.
+__device__ __forceinline__ float hue_degrees(float b, float a)
+{
+    const float kDeg = 57.295779513082321f;      // degrees per radian
+    float h = (a == 0.0f && b == 0.0f) ? 0.0f : atan2f(b, a) * kDeg;
+    if (h < 0.0f) h += 360.0f;
+    return h;
+}
+
 // CIEDE2000 with kL = kC = kH = 1, angles in degrees.
 __device__ __forceinline__ float ciede2000(float3 p, float3 q)
 {
-    const float kDeg = 57.295779513082321f;      // degrees per radian
     const float k25p7 = 6103515625.0f;
     float c1 = sqrtf(p.y * p.y + p.z * p.z);
     float c2 = sqrtf(q.y * q.y + q.z * q.z);
@@ -74,10 +82,7 @@ __device__ __forceinline__ float ciede2000(float3 p, float3 q)
     float g = 0.5f * (1.0f - sqrtf(__fdividef(cm7, cm7 + k25p7)));
     float ap1 = p.y * (1.0f + g), ap2 = q.y * (1.0f + g);
     float cp1 = sqrtf(ap1 * ap1 + p.z * p.z), cp2 = sqrtf(ap2 * ap2 + q.z * q.z);
-    float hp1 = (ap1 == 0.0f && p.z == 0.0f) ? 0.0f : atan2f(p.z, ap1) * kDeg;
-    float hp2 = (ap2 == 0.0f && q.z == 0.0f) ? 0.0f : atan2f(q.z, ap2) * kDeg;
-    if (hp1 < 0.0f) hp1 += 360.0f;
-    if (hp2 < 0.0f) hp2 += 360.0f;
+    const float hp1 = hue_degrees(p.z, ap1), hp2 = hue_degrees(q.z, ap2);
     float prod = cp1 * cp2;
     float dh = 0.0f, hm;
     if (prod == 0.0f) {
@@ -115,13 +120,37 @@ __device__ __forceinline__ float ciede2000(float3 p, float3 q)
 // geometry helpers (exact op order)
 // ---------------------------------------------------------------------------
 
+// fl(a / b) from rb = fl(1 / b): an estimate corrected twice by its exact
+// remainder.  Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor" (1990): with rb correctly rounded and q within one unit
+// in the last place, fl(q + fl(a - b q) rb) is the correctly rounded quotient;
+// the first correction brings q there.  Holds while nothing underflows or
+// overflows: kDivLo < |a| < kDivHi (or a = 0) and kDivLo < b < kDivHi.  Five
+// operations against some nineteen issue slots of __fdiv_rn.
+constexpr float kDivLo = 8.6736174e-19f, kDivHi = 1.1529215e18f;       // 2^-60, 2^60
+
+__device__ __forceinline__ float div_by(float a, float b, float rb)
+{
+    float q = __fmul_rn(a, rb);
+    q = __fmaf_rn(__fmaf_rn(-b, q, a), rb, q);
+    return __fmaf_rn(__fmaf_rn(-b, q, a), rb, q);
+}
+
+// Quotients outside that range (rare, kept out of line).
+__device__ __noinline__ float div_any(float a, float b) { return __fdiv_rn(a, b); }
+
+__device__ __forceinline__ bool div_fits(float a) { return (fabsf(a) > kDivLo && fabsf(a) < kDivHi) || a == 0.0f; }
+
 // Back-projection of pixel (u,v) at integer depth d (0.1 mm units), Sec. IV-A.
+// sc.rfx, sc.rfy: fl(1 / fx), fl(1 / fy), or 0 when fx or fy is out of div_by's range.
 __device__ __forceinline__ float3 back_project(const DevScene& sc, int u, int v, unsigned d)
 {
-    float z = __fdiv_rn(__uint2float_rn(d), 10000.0f);
-    float x = __fdiv_rn(__fmul_rn(__fsub_rn(__int2float_rn(u), sc.cx), z), sc.fx);
-    float y = __fdiv_rn(__fmul_rn(__fsub_rn(__int2float_rn(v), sc.cy), z), sc.fy);
-    return make_float3(x, y, z);
+    const float z = div_by(__uint2float_rn(d), 10000.0f, 1.0f / 10000.0f);
+    const float ax = __fmul_rn(__fsub_rn(__int2float_rn(u), sc.cx), z);
+    const float ay = __fmul_rn(__fsub_rn(__int2float_rn(v), sc.cy), z);
+    if (sc.rfx != 0.0f && div_fits(ax) && div_fits(ay))
+        return make_float3(div_by(ax, sc.fx, sc.rfx), div_by(ay, sc.fy, sc.rfy), z);
+    return make_float3(div_any(ax, sc.fx), div_any(ay, sc.fy), z);
 }
 
 // Hash-cell coordinate floor(x / cell), taken as floor(fl(x * fl(1 / cell))):
@@ -471,15 +500,18 @@ struct TriSetup {
     int A;                        // doubled area > 0
 };
 
-struct __align__(16) TriStage {   // a set-up triangle staged for its warp (64 bytes, 4 x 16-byte moves)
-    // edge i at the sample of pixel (u, v): a[i] u + b[i] v + c[i] + bias_i
-    // (two's-complement arithmetic, exact), bias_i = 1 unless edge i owns
-    // the samples lying on it; covered iff every a[i] u + b[i] v + c[i] >= 0
-    int a[3], b[3], c[3];
-    float iz[3];                  // 1/Z
-    int A, tri;                   // doubled area, triangle id
-    int uv0;                      // pixel box origin u0 | v0 << 16
-    int bw_bias;                  // box width | bias bits << 16
+// A set-up triangle staged for its warp (48 bytes, 3 x 16-byte moves): the values
+// of edges 0 and 1 at its pixel box's first sample, less their tie bias, and
+// their increments per column (a) and row (b); edge 2 holds the rest of K.  Its
+// items, numbered from `first`, are the samples of the box or, when thin, its
+// rows.
+struct __align__(16) TriStage {
+    int a0, a1, b0, b1;
+    int t0, t1, K, tri;
+    unsigned idx;                 // z-buffer index of the first sample | its flags (DepthItem) | thin << 18
+    int bw;                       // box width
+    float rbw;                    // fl(1 / bw)
+    int first;
 };
 
 __device__ __forceinline__ int edge_fn(int ax, int ay, int bx, int by, int px, int py)
@@ -494,14 +526,6 @@ __device__ __forceinline__ bool owns(int dx, int dy)
 
 __device__ __forceinline__ int floor16(int x) { return x >> 4; }         // arithmetic shift
 __device__ __forceinline__ int ceil16(int x) { return -((-x) >> 4); }
-
-// Bit i set iff edge i of the oriented triangle (edge 0: vertex 1 -> 2, edge
-// 1: 2 -> 0, edge 2: 0 -> 1) owns the samples lying on it.
-__device__ __forceinline__ int owns_of(const TriSetup& o)
-{
-    return (owns(o.x[2] - o.x[1], o.y[2] - o.y[1]) ? 1 : 0) | (owns(o.x[0] - o.x[2], o.y[0] - o.y[2]) ? 2 : 0) |
-           (owns(o.x[1] - o.x[0], o.y[1] - o.y[0]) ? 4 : 0);
-}
 
 // Doubled area and orientation of a loaded triangle: a negative area swaps
 // vertices 1 and 2 (two-sided rendering).  False if degenerate (A == 0).
@@ -522,15 +546,16 @@ __device__ __forceinline__ bool orient_triangle(TriSetup& o)
 
 // Triangle loaded at a pose: transform, near/guard-band cull, projection,
 // 4-bit snap (orient_triangle completes the set-up).  False if culled.
-__device__ __forceinline__ bool load_triangle(const DevScene& sc, const DevMesh& m,
-                                              const float* P, int4 tv, TriSetup& o)
+// (C: a DevScene, or what the rasteriser keeps of one.)
+template <class C>
+__device__ __forceinline__ bool load_triangle(const C& sc, const float4* verts, const float* P, int4 tv, TriSetup& o)
 {
     int vids[3] = {tv.x, tv.y, tv.z};
     const float gx0 = (float)(-16 * sc.W), gx1 = (float)(32 * sc.W);
     const float gy0 = (float)(-16 * sc.H), gy1 = (float)(32 * sc.H);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        float4 v = __ldg(&m.verts[vids[k]]);
+        float4 v = __ldg(&verts[vids[k]]);
         float X = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(P[0], v.x), __fmul_rn(P[1], v.y)),
                                       __fmul_rn(P[2], v.z)), P[3]);
         float Y = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(P[4], v.x), __fmul_rn(P[5], v.y)),
@@ -548,24 +573,6 @@ __device__ __forceinline__ bool load_triangle(const DevScene& sc, const DevMesh&
         o.vid[k] = vids[k];
     }
     return true;
-}
-
-// Depth of a covered sample from the edge values (perspective-correct:
-// z = A / (w0/Z0 + w1/Z1 + w2/Z2), one division).
-// Returns false if the depth falls outside [1, 2^32-1].
-__device__ __forceinline__ bool sample_depth(int w0, int w1, int w2, const float* iz, int A,
-                                             unsigned& d)
-{
-    float num = __fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(w0), iz[0]),
-                                    __fmul_rn(__int2float_rn(w1), iz[1])),
-                          __fmul_rn(__int2float_rn(w2), iz[2]));
-    float z = __fdiv_rn(__int2float_rn(A), num);
-    float dz = __fmul_rn(z, 10000.0f);
-    // z >= 0 here (A > 0 and every 1/Z > 0), so dz in [0, 2^32) rounds to
-    // nearest in 32 bits (the largest binary32 below 2^32 is an integer)
-    if (!(dz < 4294967296.0f)) return false;
-    d = __float2uint_rn(dz);
-    return d >= 1u;
 }
 
 template <bool K32>
@@ -609,18 +616,19 @@ struct __align__(16) WarpProbe {
                                   // dense index: runs[r].x of the non-empty rows
     int total;                    // hash: candidates of the group's 27 cells
     unsigned char qlist[32];      // hash: the lanes of the group's queries, in lane order
-    float4 q[32];                 // query of each lane (dense index: -x, -x, -y, -y)
+    float4 q[32];                 // the group's queries as -x, -x, -y, -y (hash: the query of each lane)
     unsigned long long best[32];  // hash: nearest-neighbour key of each lane's query
     float4 stage[64];             // hash: a chunk of the group's candidates, shared by its queries;
-                                  // dense index: .xy = -z, -z of each lane's query
+                                  // dense index: .xyz = -z, -z, pixel of the group's queries
 };
 
 // Per-warp scratch: the radius search and the rasteriser's triangle stage
 // use the same bytes (the two phases are separated by block barriers).
-constexpr size_t kWarpScratch = sizeof(WarpProbe) > 32 * sizeof(TriStage) ? sizeof(WarpProbe)
-                                                                            : 32 * sizeof(TriStage);
+constexpr size_t kRasterScratch = 64 * sizeof(uint4) + 21 * sizeof(TriStage);   // its triangle ring and staged triangles
+constexpr size_t kWarpScratch = sizeof(WarpProbe) > kRasterScratch ? sizeof(WarpProbe) : kRasterScratch;
+static_assert(kWarpQueue * sizeof(float4) >= 64 * 16, "the depth ring fits the kept-point queue it aliases");
 static_assert(sizeof(KeptPoint) == 16, "kept-point queue entries are 16 bytes");
-static_assert(sizeof(TriStage) == 64, "staged triangles are 64 bytes");
+static_assert(sizeof(TriStage) == 48, "staged triangles are 48 bytes");
 static_assert(kWarpScratch % 16 == 0, "per-warp scratch keeps 16-byte alignment");
 static_assert(sizeof(WarpProbe) % 16 == 0, "per-warp scratch keeps 16-byte alignment");
 
@@ -849,17 +857,19 @@ __device__ __forceinline__ float4 group_candidate(const DevScene& sc, const int2
     float4 p = make_float4(far, far, far, 0.0f);
     const unsigned rel = (unsigned)(off - c);
     const unsigned starts = __reduce_or_sync(0xffffffffu, cnt != 0 && rel < 32u ? 1u << rel : 0u);
+    begun += __popc(starts & (0xffffffffu >> (31 - lane)));
     if (c + lane < T) {
         // the candidate lies in the last row begun at or before it
-        const int i = base[begun + __popc(starts & (0xffffffffu >> (31 - lane))) - 1].x + c + lane;
+        const int i = base[begun - 1].x + c + lane;
         if (PERCH_CHECKED((unsigned)i < (unsigned)sc.n_pts, err)) p = __ldg(&sc.pts[i]);
     }
-    begun += __popc(starts);
+    begun = __shfl_sync(0xffffffffu, begun, 31);
     return p;
 }
 
 // Radius search of up to 32 points through the dense cell index.  Lanes whose
-// points fall in the same cell form a group.  The group's candidates -- nine
+// points fall in the same cell form a group; the groups are taken in order of
+// their cells.  A group's candidates -- nine
 // rows of three cells, each row one run of the cell-sorted points -- are held
 // two or four per lane in registers, loaded once by coalesced reads; every
 // query of the group is then broadcast to them, and the warp's minimum of the
@@ -870,12 +880,13 @@ __device__ __forceinline__ float4 group_candidate(const DevScene& sc, const int2
 // delta; only the ends of the whole index are clamped.  NEAR: the caller has
 // tested the near-cell bits.
 //
-// Bound by instruction issue.  A group costs about 70 instructions, a query
-// about 20 per 64 candidates (30 per 128), against the 16 to 230 candidates of
-// a mean query on the tabletop and 6-DoF scenes.  Staging the candidates in
-// shared memory and splitting the lanes over the group's queries cost about
-// twice that: three 640x480 objects x 29,584 poses 45.2 -> 42.0 ms, five 6-DoF
-// objects x 4,096 poses 27.9 -> 22.8 ms, their refinement 52.3 -> 42.7 ms.
+// Bound by instruction issue: about 90 instructions a group and 30 a query per 64
+// candidates (45 per 128), against the 16 to 230 candidates of a mean query on
+// the tabletop and 6-DoF scenes.  Staging the candidates in shared memory and
+// splitting the lanes over the group's queries costs about half as much again
+// (155k against 105k warp instructions per pose of an ellipsoid, 771k against
+// 487k per 6-DoF pose), and four lanes per query walking its nine rows alone
+// 142k and 628k: the longest row of eight queries counts for all of them.
 template <bool MARK, bool NEAR>
 __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bool valid, float4 query, WarpProbe& W,
                                                           int lane, const MarkBand& mb)
@@ -891,19 +902,23 @@ __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bo
             if (NEAR || ((__ldg(&sc.near_bits[c >> 5]) >> (c & 31)) & 1u)) cell = c;
         }
     }
-    W.q[lane] = make_float4(-query.x, -query.x, -query.y, -query.y);
-    W.stage[lane] = make_float4(-query.z, -query.z, query.w, 0.0f);
-    const unsigned grp = __match_any_sync(0xffffffffu, cell);
+    const unsigned lt = (1u << lane) - 1u;
     const unsigned d2max = __float_as_uint(sc.delta2);
     // lane j < 9: from a cell to the first of the three cells of its row j
     const int row_off = (lane % 3 - 1) * nx + (lane / 3 - 1) * nxy - 1;
     unsigned bd = 0xFFFFFFFFu, bp = 0xFFFFFFFFu;          // the lane's own nearest point
-    __syncwarp();
-    for (unsigned rest = __ballot_sync(0xffffffffu, cell >= 0 && (grp & ((1u << lane) - 1u)) == 0u); rest != 0;
-         rest &= rest - 1) {
-        const int L = __ffs(rest) - 1;
-        const int c = __shfl_sync(0xffffffffu, cell, L);
-        const unsigned members = __shfl_sync(0xffffffffu, grp, L);
+    for (;;) {
+        // the lowest cell not yet searched (-1, none, is the largest unsigned)
+        const int c = (int)__reduce_min_sync(0xffffffffu, (unsigned)cell);
+        if (c < 0) break;
+        const bool mine = cell == c;
+        const unsigned members = __ballot_sync(0xffffffffu, mine);
+        const int G = __popc(members), pos = mine ? __popc(members & lt) : -1;
+        if (mine) {
+            cell = -1;
+            W.q[pos] = make_float4(-query.x, -query.x, -query.y, -query.y);
+            W.stage[pos] = make_float4(-query.z, -query.z, query.w, 0.0f);
+        }
         int s0 = 0, cnt = 0;
         if (lane < 9) {
             s0 = (int)__ldg(&sc.cell_start[min(max(c + row_off, 0), ncell)]);
@@ -918,17 +933,18 @@ __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bo
         const int T = __shfl_sync(0xffffffffu, off, 8);
         off -= cnt;
         const unsigned nonempty = __ballot_sync(0xffffffffu, cnt != 0);
-        if (cnt != 0) W.runs[__popc(nonempty & ((1u << lane) - 1u))].x = s0 - off;
+        if (cnt != 0) W.runs[__popc(nonempty & lt)].x = s0 - off;
         __syncwarp();
         int begun = 0;
+#pragma unroll 1
         for (int c0 = 0; c0 < T; c0 += 128) {
             const float4 ca = group_candidate(sc, W.runs, off, cnt, c0, T, lane, begun, mb.err);
             const float4 cb = group_candidate(sc, W.runs, off, cnt, c0 + 32, T, lane, begun, mb.err);
             const unsigned long long x0 = pack2(ca.x, cb.x), y0 = pack2(ca.y, cb.y), z0 = pack2(ca.z, cb.z);
             const unsigned pa = __float_as_uint(ca.w), pb = __float_as_uint(cb.w);
             if (T - c0 <= 64) {
-                for (unsigned m = members; m != 0; m &= m - 1) {
-                    const int i = __ffs(m) - 1;
+#pragma unroll 1
+                for (int i = 0; i < G; ++i) {
                     const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&W.q[i]);
                     const unsigned long long qz = *reinterpret_cast<const unsigned long long*>(&W.stage[i]);
                     const uint2 d = dist2_pair(qa, qz, x0, y0, z0);
@@ -941,7 +957,7 @@ __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bo
                     if (dm > d2max) continue;
                     const unsigned pm = __reduce_min_sync(
                         0xffffffffu, min(d.x == dm ? pa : 0xFFFFFFFFu, d.y == dm ? pb : 0xFFFFFFFFu));
-                    if (lane == i && (dm < bd || (dm == bd && pm < bp))) {
+                    if (pos == i && (dm < bd || (dm == bd && pm < bp))) {
                         bd = dm;
                         bp = pm;
                     }
@@ -951,8 +967,8 @@ __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bo
                 const float4 cd = group_candidate(sc, W.runs, off, cnt, c0 + 96, T, lane, begun, mb.err);
                 const unsigned long long x1 = pack2(cc.x, cd.x), y1 = pack2(cc.y, cd.y), z1 = pack2(cc.z, cd.z);
                 const unsigned pc = __float_as_uint(cc.w), pd = __float_as_uint(cd.w);
-                for (unsigned m = members; m != 0; m &= m - 1) {
-                    const int i = __ffs(m) - 1;
+#pragma unroll 1
+                for (int i = 0; i < G; ++i) {
                     const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&W.q[i]);
                     const unsigned long long qz = *reinterpret_cast<const unsigned long long*>(&W.stage[i]);
                     const uint2 d = dist2_pair(qa, qz, x0, y0, z0), e = dist2_pair(qa, qz, x1, y1, z1);
@@ -968,7 +984,7 @@ __device__ __forceinline__ unsigned long long probe_dense(const DevScene& sc, bo
                     const unsigned pm = __reduce_min_sync(
                         0xffffffffu, min(min(d.x == dm ? pa : 0xFFFFFFFFu, d.y == dm ? pb : 0xFFFFFFFFu),
                                          min(e.x == dm ? pc : 0xFFFFFFFFu, e.y == dm ? pd : 0xFFFFFFFFu)));
-                    if (lane == i && (dm < bd || (dm == bd && pm < bp))) {
+                    if (pos == i && (dm < bd || (dm == bd && pm < bp))) {
                         bd = dm;
                         bp = pm;
                     }
@@ -995,62 +1011,72 @@ __device__ __forceinline__ unsigned long long probe_batch(const DevScene& sc, bo
 // Conservative pixel box of an object-frame box [lo,hi] at pose P (2 px
 // margin), clipped to [cu0,cu1) x [cv0,cv1).  Falls back to the clip box
 // when a corner is not in front of the camera.  Also returns the largest Z.
-__device__ void project_box(const DevScene& sc, const float* P, const float* lo, const float* hi,
-                            int cu0, int cv0, int cu1, int cv1, int* box, float* zmax)
+// A whole warp calls it, corner c in lanes c, c + 8, ...: one corner's latency
+// instead of eight, and a fraction of the code (the kernel's loops compete for
+// the instruction cache, so it is also called, not inlined).
+struct PixelBox {
+    int4 box;
+    float zmax;
+};
+
+__device__ __noinline__ PixelBox project_box(float4 camera, const float* P, float3 lo, float3 hi, int4 clip)
 {
-    float umin = 3.0e38f, umax = -3.0e38f, vmin = 3.0e38f, vmax = -3.0e38f, zm = -3.0e38f;
-    bool ok = true;
-    for (int c = 0; c < 8; ++c) {
-        float x = (c & 1) ? hi[0] : lo[0];
-        float y = (c & 2) ? hi[1] : lo[1];
-        float z = (c & 4) ? hi[2] : lo[2];
-        float X = P[0] * x + P[1] * y + P[2] * z + P[3];
-        float Y = P[4] * x + P[5] * y + P[6] * z + P[7];
-        float Z = P[8] * x + P[9] * y + P[10] * z + P[11];
-        zm = fmaxf(zm, Z);
-        if (!(Z > 1e-4f)) {
-            ok = false;
-            continue;
-        }
-        float u = sc.fx * (X / Z) + sc.cx, v = sc.fy * (Y / Z) + sc.cy;
+    const int lane = threadIdx.x & 31;
+    const float x = (lane & 1) ? hi.x : lo.x;
+    const float y = (lane & 2) ? hi.y : lo.y;
+    const float z = (lane & 4) ? hi.z : lo.z;
+    const float X = P[0] * x + P[1] * y + P[2] * z + P[3];
+    const float Y = P[4] * x + P[5] * y + P[6] * z + P[7];
+    const float Z = P[8] * x + P[9] * y + P[10] * z + P[11];
+    float zm = fmaxf(-3.0e38f, Z), umin = 3.0e38f, umax = -3.0e38f, vmin = 3.0e38f, vmax = -3.0e38f;
+    const bool front = Z > 1e-4f;
+    if (front) {
+        const float u = camera.x * div_any(X, Z) + camera.z, v = camera.y * div_any(Y, Z) + camera.w;
         umin = fminf(umin, u); umax = fmaxf(umax, u);
         vmin = fminf(vmin, v); vmax = fmaxf(vmax, v);
     }
-    *zmax = zm;
-    if (!ok || !(umax - umin < 1.0e7f) || !(vmax - vmin < 1.0e7f)) {
-        box[0] = cu0; box[1] = cv0; box[2] = cu1; box[3] = cv1;
-        return;
+#pragma unroll 1
+    for (int o = 4; o > 0; o >>= 1) {
+        zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
+        umin = fminf(umin, __shfl_xor_sync(0xffffffffu, umin, o));
+        umax = fmaxf(umax, __shfl_xor_sync(0xffffffffu, umax, o));
+        vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
+        vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
     }
-    int u0 = (int)floorf(fmaxf(umin, -1.0e7f)) - 2, u1 = (int)ceilf(fminf(umax, 1.0e7f)) + 3;
-    int v0 = (int)floorf(fmaxf(vmin, -1.0e7f)) - 2, v1 = (int)ceilf(fminf(vmax, 1.0e7f)) + 3;
-    box[0] = max(u0, cu0); box[1] = max(v0, cv0);
-    box[2] = min(u1, cu1); box[3] = min(v1, cv1);
-    if (box[2] < box[0]) box[2] = box[0];
-    if (box[3] < box[1]) box[3] = box[1];
+    const bool ok = __ballot_sync(0xffffffffu, !front) == 0u;
+    PixelBox r = {clip, zm};
+    if (ok && umax - umin < 1.0e7f && vmax - vmin < 1.0e7f) {
+        const int u0 = (int)floorf(fmaxf(umin, -1.0e7f)) - 2, u1 = (int)ceilf(fminf(umax, 1.0e7f)) + 3;
+        const int v0 = (int)floorf(fmaxf(vmin, -1.0e7f)) - 2, v1 = (int)ceilf(fminf(vmax, 1.0e7f)) + 3;
+        r.box.x = max(u0, clip.x);
+        r.box.y = max(v0, clip.y);
+        r.box.z = max(min(u1, clip.z), r.box.x);
+        r.box.w = max(min(v1, clip.w), r.box.y);
+    }
+    return r;
 }
 
 // Shared-memory carve-up of one scoring block.
 struct ScoreSmem {
-    uint32_t* zbuf;               // z-buffer tile (32- or 64-bit keys)
+    uint32_t* zbuf;               // z-buffer tile (32- or 64-bit keys), at offset 0
     uint32_t* marks;              // admissible-band bitset
-    KeptPoint* kept;              // per warp: resolve -> radius-search ring queue
-    WarpProbe* probe;             // per warp scratch of the radius search (aliases stage)
-    TriStage* stage;              // per warp 32 staged triangles (aliases probe)
     int* next_batch;
     int* refused;                 // tree edges: the object would occlude a placed one
     int* bin_cnt;                 // kBinTiles: triangles binned per z-buffer tile
     int* jo_next;                 // plain scoring: next chunk of J_o's |I cap V|
-    int* raster_done;             // plain scoring: warps done with the tile's raster
     int* vbounds;                 // snapped vertex bounds of the hypothesis (vertex_pass)
 };
 
 // ---- per-hypothesis vertex cache (one slot of global scratch per block) ----
 //
 // Each vertex is transformed, projected and snapped once per hypothesis and
-// kept as (x16 : int16, y16 : int16, 1/Z : float); a vertex that fails the
-// near-plane or guard-band test is stored with x16 = -32768, which culls every
-// triangle that uses it.  Used when 32 W and 32 H fit in int16.
-constexpr int kCulledX = -32768;
+// kept as (x16, y16 : unsigned 16 bits, biased by kSnapBias, 1/Z : float), so
+// that a triangle's box comes from packed unsigned minima and maxima; a vertex
+// that fails the near-plane or guard-band test is stored as x16 = y16 = 0xFFFF,
+// which culls every triangle that uses it.  Used when W and H are at most 1023
+// (snapped coordinates in [-16 x 1023, 32 x 1023)).
+constexpr int kSnapBias = 1 << 14;            // 1024 pixels in 1/16 px
+constexpr uint32_t kCulledXY = 0xFFFFFFFFu;
 
 //
 // bounds (optional, shared memory, initialised to INT_MAX, INT_MAX, INT_MIN,
@@ -1061,7 +1087,7 @@ __device__ __forceinline__ void vertex_pass(const DevScene& sc, const DevMesh& m
     const float gx0 = (float)(-16 * sc.W), gx1 = (float)(32 * sc.W);
     const float gy0 = (float)(-16 * sc.H), gy1 = (float)(32 * sc.H);
     int xmin = INT_MAX, ymin = INT_MAX, xmax = INT_MIN, ymax = INT_MIN;
-#pragma unroll 2
+#pragma unroll 1
     for (int i = threadIdx.x; i < m.n_verts; i += nt) {
         float4 v = __ldg(&m.verts[i]);
         float X = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(P[0], v.x), __fmul_rn(P[1], v.y)),
@@ -1070,18 +1096,25 @@ __device__ __forceinline__ void vertex_pass(const DevScene& sc, const DevMesh& m
                                       __fmul_rn(P[6], v.z)), P[7]);
         float Z = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(P[8], v.x), __fmul_rn(P[9], v.y)),
                                       __fmul_rn(P[10], v.z)), P[11]);
-        unsigned long long rec = (unsigned long long)(uint16_t)kCulledX;
+        unsigned long long rec = kCulledXY;
         if (Z >= sc.z_near) {
-            float sx = __fmul_rn(__fadd_rn(__fmul_rn(sc.fx, __fdiv_rn(X, Z)), sc.cx), 16.0f);
-            float sy = __fmul_rn(__fadd_rn(__fmul_rn(sc.fy, __fdiv_rn(Y, Z)), sc.cy), 16.0f);
+            const float iz = __frcp_rn(Z);
+            float xz, yz;
+            if (div_fits(X) && div_fits(Y) && Z > kDivLo && Z < kDivHi) {
+                xz = div_by(X, Z, iz);
+                yz = div_by(Y, Z, iz);
+            } else {
+                xz = div_any(X, Z);
+                yz = div_any(Y, Z);
+            }
+            const float sx = __fmul_rn(__fadd_rn(__fmul_rn(sc.fx, xz), sc.cx), 16.0f);
+            const float sy = __fmul_rn(__fadd_rn(__fmul_rn(sc.fy, yz), sc.cy), 16.0f);
             if (sx >= gx0 && sx < gx1 && sy >= gy0 && sy < gy1) {
                 const int xi = __float2int_rn(sx), yi = __float2int_rn(sy);
                 xmin = min(xmin, xi); xmax = max(xmax, xi);
                 ymin = min(ymin, yi); ymax = max(ymax, yi);
-                uint32_t xs = (uint16_t)(int16_t)xi;
-                uint32_t ys = (uint16_t)(int16_t)yi;
-                rec = (unsigned long long)(xs | (ys << 16)) |
-                      ((unsigned long long)__float_as_uint(__frcp_rn(Z)) << 32);
+                rec = (unsigned long long)((uint32_t)(xi + kSnapBias) | ((uint32_t)(yi + kSnapBias) << 16)) |
+                      ((unsigned long long)__float_as_uint(iz) << 32);
             }
         }
         vc[i] = rec;
@@ -1110,10 +1143,9 @@ __device__ __forceinline__ bool load_cached(const unsigned long long* vc, int4 t
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const unsigned long long r = rec[k];
-        const int xs = (int16_t)(uint16_t)(r & 0xFFFFu);
-        ok = ok && xs != kCulledX;
-        o.x[k] = xs;
-        o.y[k] = (int16_t)(uint16_t)((r >> 16) & 0xFFFFu);
+        ok = ok && (uint32_t)r != kCulledXY;
+        o.x[k] = (int)(r & 0xFFFFu) - kSnapBias;
+        o.y[k] = (int)((r >> 16) & 0xFFFFu) - kSnapBias;
         o.iz[k] = __uint_as_float((uint32_t)(r >> 32));
         o.vid[k] = vids[k];
     }
@@ -1127,7 +1159,7 @@ __device__ __forceinline__ bool load_tri(const DevScene& sc, const DevMesh& m, c
                                          const unsigned long long* vc, int4 tv, TriSetup& o)
 {
     if (VC) return load_cached(vc, tv, o);
-    return load_triangle(sc, m, P, tv, o);
+    return load_triangle(sc, m.verts, P, tv, o);
 }
 
 // Full set-up of triangle t at pose P: load, then orientation.  False if
@@ -1149,177 +1181,325 @@ __device__ __forceinline__ int div_small(int n, int d)
     return q;
 }
 
-// Coverage (edge functions and the ownership rule), depth and the z-buffer
-// update of sample (u, v) of a set-up triangle (vertices in 1/16 px, 1/Z,
-// doubled area A > 0, owns bits per edge), in the tile at (tu0, tv0).
-template <bool K32>
-__device__ __forceinline__ void raster_sample(const int* x, const int* y, const float* iz, int A, int owns_bits,
-                                              int tri, int u, int v, uint32_t* zbuf, int tu0, int tv0, int tw,
-                                              int tcap, float izmax, int* err)
-{
-    const int idx = (v - tv0) * tw + (u - tu0);
-    if (!PERCH_CHECKED((unsigned)idx < (unsigned)tcap, err)) return;
-    // Early out for a sample that cannot beat the depth already stored here:
-    // its depth is at least 1e4 / max(1/Z) less a few 2^-24 relative, so if
-    // max(1/Z) (d_here + 2) < 9999 its depth is at least d_here + 2 and its
-    // key is larger.  The stored key only decreases, so reading it while other
-    // samples update it can only make this test skip less.
-    {
-        unsigned dh;
-        if (K32) {
-            const uint32_t w = zbuf[idx];
-            dh = w == 0xFFFFFFFFu ? 0xFFFFFFFFu : (w >> 16);
-        } else {
-            const unsigned long long w = reinterpret_cast<const unsigned long long*>(zbuf)[idx];
-            dh = w == kEmptyKey ? 0xFFFFFFFFu : (unsigned)(w >> 32);
-        }
-        if (dh < 0xFFFFFFF0u && __fmul_rn(izmax, __uint2float_rn(dh + 2u)) < 9999.0f) return;
-    }
-    const int sx = 16 * u, sy = 16 * v;
-    const int w0 = edge_fn(x[1], y[1], x[2], y[2], sx, sy);
-    const int w1 = edge_fn(x[2], y[2], x[0], y[0], sx, sy);
-    const int w2 = edge_fn(x[0], y[0], x[1], y[1], sx, sy);
-    const bool cov = (w0 > 0 || (w0 == 0 && (owns_bits & 1))) &&
-                     (w1 > 0 || (w1 == 0 && (owns_bits & 2))) &&
-                     (w2 > 0 || (w2 == 0 && (owns_bits & 4)));
-    unsigned d;
-    if (cov && sample_depth(w0, w1, w2, iz, A, d)) zmin<K32>(zbuf, idx, d, tri, err);
-}
-
-// Coverage, depth and the z-buffer update of sample (u, v) of a staged
-// triangle: the same tests as raster_sample from the edge coefficients (no
-// vertex differences per sample), coverage first so that an uncovered sample
-// reads no z-buffer word.
-template <bool K32>
-__device__ __forceinline__ void raster_staged(const TriStage& e, int u, int v, uint32_t* zbuf, int tu0, int tv0,
-                                              int tw, int tcap, int* err)
-{
-    const int t0 = (int)((unsigned)e.a[0] * (unsigned)u + (unsigned)e.b[0] * (unsigned)v + (unsigned)e.c[0]);
-    const int t1 = (int)((unsigned)e.a[1] * (unsigned)u + (unsigned)e.b[1] * (unsigned)v + (unsigned)e.c[1]);
-    const int t2 = (int)((unsigned)e.a[2] * (unsigned)u + (unsigned)e.b[2] * (unsigned)v + (unsigned)e.c[2]);
-    if ((t0 | t1 | t2) < 0) return;
-    const int idx = (v - tv0) * tw + (u - tu0);
-    if (!PERCH_CHECKED((unsigned)idx < (unsigned)tcap, err)) return;
-    {   // the early out of raster_sample
-        const float izmax = fmaxf(e.iz[0], fmaxf(e.iz[1], e.iz[2]));
-        unsigned dh;
-        if (K32) {
-            const uint32_t w = zbuf[idx];
-            dh = w == 0xFFFFFFFFu ? 0xFFFFFFFFu : (w >> 16);
-        } else {
-            const unsigned long long w = reinterpret_cast<const unsigned long long*>(zbuf)[idx];
-            dh = w == kEmptyKey ? 0xFFFFFFFFu : (unsigned)(w >> 32);
-        }
-        if (dh < 0xFFFFFFF0u && __fmul_rn(izmax, __uint2float_rn(dh + 2u)) < 9999.0f) return;
-    }
-    const int bias = e.bw_bias >> 16;
-    unsigned d;
-    if (sample_depth(t0 + (bias & 1), t1 + ((bias >> 1) & 1), t2 + (bias >> 2), e.iz, e.A, d))
-        zmin<K32>(zbuf, idx, d, e.tri, err);
-}
-
-// Rasterise every triangle of mesh m at pose P into the z-buffer tile
-// [tu0,tu1) x [tv0,tv1) (row pitch tw).  A warp sets up 32 triangles (one per
-// lane); a triangle with one sample in its box is tested in its own lane, the
-// others are staged in shared memory (TS, 32 entries per warp) and the
-// samples of their boxes spread evenly over the lanes (a prefix sum of the box
-// areas, then a binary search per sample for its triangle).  No barrier inside.
+// ---- rasteriser: rings of triangles and covered samples --------------------
 //
-// LIST: the triangles are list[0 .. n_list) (the tile's bin, written by this
-// block) instead of the whole mesh.
-template <int NT, bool K32, bool VC, bool LIST = false>
-__device__ __forceinline__ void raster_tile(const DevScene& sc, const DevMesh& mesh, const float* P,
-                                            const unsigned long long* vc, TriStage* TS, uint32_t* zbuf,
-                                            int tu0, int tv0, int tu1, int tv1, int tw, int* err,
-                                            const int* list = nullptr, int n_list = 0)
+// A fine mesh leaves few lanes of a warp anything to do at a time: a third to a
+// half of its triangles hold no sample, and about one sample in four that is
+// tested is covered.  So the triangles whose boxes hold samples are queued in
+// shared memory and set up by 32 full lanes, and the covered samples are queued
+// again until 32 of them can have their depth (a division) and z-buffer update.
+constexpr int kRing = 64;         // entries of a warp's ring of triangles or samples
+constexpr int kStaged = 21;       // larger triangles expanded at a time (the scratch's size)
+constexpr int kTinyBox = 8;       // boxes of up to this many samples are walked in one lane
+
+// A covered sample: edges 0 and 1 less their tie bias, the triangle, and the
+// z-buffer index with the biases in bits 16 and 17.
+struct __align__(16) DepthItem {
+    int t0, t1, tri;
+    unsigned idx;
+};
+
+extern __shared__ __align__(16) unsigned char g_smem[];
+
+// The rasteriser's arguments, by value: it is called, not inlined, so that its
+// loops have the registers to themselves (inlined, they ran from spilled
+// values).  Shared-memory places are byte offsets from the block's base, so that
+// every access is a shared-memory one.
+struct RasterArgs {
+    const int4* tris;
+    const unsigned long long* vc; // vertex cache, or nullptr: vertices transformed again (cam)
+    const int* list;              // the tile's bin, or nullptr: triangles 0 .. n - 1
+    int n;
+    int tu0, tv0, tu1, tv1, tw;   // tile [tu0,tu1) x [tv0,tv1), row pitch tw
+    unsigned scratch, ring;       // the warp's triangle ring and staged triangles; its depth ring
+    int* err;
+};
+
+struct RasterCamera {             // without the vertex cache
+    const float4* verts;
+    const float* P;
+    int W, H;
+    float fx, fy, cx, cy, z_near;
+};
+
+// Depth and z-buffer update of the n <= 32 oldest samples of the ring at `at`:
+// the triangle is read again (its weights and 1/Z in the orientation's order),
+// z = A / ((w0/Z0 + w1/Z1) + w2/Z2) with one division, d = rint(10000 z).
+template <bool K32, bool VC>
+__device__ __forceinline__ void depth_flush(const RasterArgs& a, const RasterCamera& cam, int at, int n, int lane)
+{
+    __syncwarp();
+    if (lane < n) {
+        const DepthItem e = reinterpret_cast<const DepthItem*>(g_smem + a.ring)[(at + lane) & (kRing - 1)];
+        const int4 tv = __ldg(&a.tris[e.tri]);
+        TriSetup o;
+        if (VC) load_cached(a.vc, tv, o);
+        else load_triangle(cam, cam.verts, cam.P, tv, o);
+        const int A = edge_fn(o.x[0], o.y[0], o.x[1], o.y[1], o.x[2], o.y[2]);
+        const int idx = (int)(e.idx & 0xFFFFu);
+        const int w0 = e.t0 + (int)((e.idx >> 16) & 1u), wa = e.t1 + (int)((e.idx >> 17) & 1u);
+        const int wb = (int)((unsigned)abs(A) - (unsigned)w0 - (unsigned)wa);
+        // a triangle of negative area has its vertices 1 and 2 exchanged
+        const float f1 = __fmul_rn(__int2float_rn(wa), o.iz[1]), f2 = __fmul_rn(__int2float_rn(wb), o.iz[2]);
+        const float f0 = __fmul_rn(__int2float_rn(w0), o.iz[0]);
+        const float num = __fadd_rn(__fadd_rn(f0, A < 0 ? f2 : f1), A < 0 ? f1 : f2);
+        const float dz = __fmul_rn(__fdiv_rn(__int2float_rn(abs(A)), num), 10000.0f);
+        // dz >= 0 (every weight and 1/Z is), so dz in [0, 2^32) rounds to
+        // nearest in 32 bits (the largest binary32 below 2^32 is an integer)
+        if (dz < 4294967296.0f && PERCH_CHECKED((unsigned)idx < (unsigned)(a.tw * (a.tv1 - a.tv0)), a.err)) {
+            const unsigned d = __float2uint_rn(dz);
+            if (d >= 1u) zmin<K32>(reinterpret_cast<uint32_t*>(g_smem), idx, d, e.tri, a.err);
+        }
+    }
+    __syncwarp();
+}
+
+// Rasterise triangles at a pose into the z-buffer tile at the start of the
+// block's shared memory.  A warp reads 32 triangles at a time and queues those
+// whose pixel box holds a sample of the tile; 32 queued ones are set up, one per
+// lane.  Boxes of up to kTinyBox samples are walked in their lanes by edge
+// increments.  Larger triangles are staged in shared memory (kStaged at a time,
+// the rest go back to the queue) and their items -- samples, or rows when the
+// triangle covers less than a quarter of its box, like the wedges of a can's end
+// caps -- spread over the lanes; a row is narrowed to the samples between the
+// edges (with a margin; coverage is still tested) and walked by its lane.
+// Covered samples go through the depth ring.  No barrier inside.
+//
+// Bound by instruction issue: the two rings keep the lanes full, and the walk,
+// the depth and the set-up each stand in the code once, because the kernel's
+// loops together are at the size of the instruction cache (a version with the
+// walk and the depth inlined three times issued fewer instructions and took 1.5
+// times as long, 5 to 9 warps in 16 waiting for instructions).  A render of a
+// 20,000-triangle ellipsoid or a 9,984-triangle can costs 127k and 122k warp
+// instructions, against 202k and 159k without the triangle ring.  With it, three
+// 640x480 objects x 29,584 poses 42.0 -> 36.2 ms, five 6-DoF objects of 30,000
+// triangles x 4,096 poses 1.41 times the former rate.
+template <int NT, bool K32, bool VC>
+__device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera cam)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int tcap = tw * (tv1 - tv0);
-    const int n = LIST ? n_list : mesh.n_tris;
-    // id and vertex ids of the lane's next triangle, loaded one iteration ahead
-    int t_next = warp * 32 + lane;
-    if (LIST && t_next < n) t_next = list[t_next];
-    int4 tv_next = warp * 32 + lane < n ? __ldg(&mesh.tris[t_next]) : make_int4(0, 0, 0, 0);
-    for (int base = warp * 32; base < n; base += NT) {
-        const int i = base + lane;
-        const int t = LIST ? t_next : i;
-        const int4 tv = tv_next;
-        if (i + NT < n) {
-            t_next = LIST ? list[i + NT] : i + NT;
-            tv_next = __ldg(&mesh.tris[t_next]);
+    const unsigned lt = (1u << lane) - 1u;
+    uint4* const TR = reinterpret_cast<uint4*>(g_smem + a.scratch);
+    TriStage* const TS = reinterpret_cast<TriStage*>(g_smem + a.scratch + kRing * sizeof(uint4));
+    DepthItem* const DQ = reinterpret_cast<DepthItem*>(g_smem + a.ring);
+    int head = 0, count = 0, dhead = 0, dcount = 0;     // the rings of triangles and samples
+    // with the vertex cache, pixels are biased like its coordinates
+    constexpr int kPix = VC ? kSnapBias / 16 : 0;
+    const uint32_t tlo = (uint32_t)(a.tu0 + kPix) | ((uint32_t)(a.tv0 + kPix) << 16);
+    const uint32_t thi = (uint32_t)(a.tu1 - 1 + kPix) | ((uint32_t)(a.tv1 - 1 + kPix) << 16);
+    // vertex ids are loaded two iterations ahead, the vertices' snapped positions
+    // (the low halves of their records) one
+    int base = warp * 32, t_next = base + lane;
+    uint4 e_next = make_uint4(0u, 0u, 0u, 0u);          // positions and id of the next triangle
+    int4 tv_next = make_int4(0, 0, 0, 0);               // vertex ids of the one after it (VC), else of the next
+    if (base + lane < a.n) {
+        if (a.list) t_next = a.list[t_next];
+        e_next.w = (unsigned)t_next;
+        tv_next = __ldg(&a.tris[t_next]);
+        if (VC) {
+            e_next.x = (uint32_t)a.vc[tv_next.x]; e_next.y = (uint32_t)a.vc[tv_next.y]; e_next.z = (uint32_t)a.vc[tv_next.z];
         }
-        int area = 0;
-        TriSetup o;
-        // the sample box does not depend on the orientation: test it first, so
-        // that the many triangles covering no sample of the tile skip the rest
-        if (i < n && load_tri<VC>(sc, mesh, P, vc, tv, o)) {
-            int xmin = min(o.x[0], min(o.x[1], o.x[2])), xmax = max(o.x[0], max(o.x[1], o.x[2]));
-            int ymin = min(o.y[0], min(o.y[1], o.y[2])), ymax = max(o.y[0], max(o.y[1], o.y[2]));
-            int u0 = max(ceil16(xmin), tu0), u1 = min(floor16(xmax), tu1 - 1);
-            int v0 = max(ceil16(ymin), tv0), v1 = min(floor16(ymax), tv1 - 1);
-            if (u0 <= u1 && v0 <= v1 && orient_triangle(o)) {
-                const int owns_bits = (owns(o.x[2] - o.x[1], o.y[2] - o.y[1]) ? 1 : 0) |
-                                      (owns(o.x[0] - o.x[2], o.y[0] - o.y[2]) ? 2 : 0) |
-                                      (owns(o.x[1] - o.x[0], o.y[1] - o.y[0]) ? 4 : 0);
-                const float izmax = fmaxf(o.iz[0], fmaxf(o.iz[1], o.iz[2]));
-                if (u0 == u1 && v0 == v1) {
-                    // one sample in the box (most triangles of a fine mesh):
-                    // test it in this lane, no staging
-                    raster_sample<K32>(o.x, o.y, o.iz, o.A, owns_bits, t, u0, v0, zbuf, tu0, tv0, tw, tcap, izmax,
-                                       err);
-                } else {
-                    area = (u1 - u0 + 1) * (v1 - v0 + 1);
-                    // edge i from vertex p to vertex q at the sample (16 u, 16 v):
-                    // (xq - xp)(16 v - yp) - (yq - yp)(16 u - xp), less its tie bias
-                    TriStage e;
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        const int p = (i + 1) % 3, q = (i + 2) % 3;
-                        const unsigned dx = (unsigned)o.x[q] - (unsigned)o.x[p];
-                        const unsigned dy = (unsigned)o.y[q] - (unsigned)o.y[p];
-                        e.a[i] = (int)(0u - 16u * dy);
-                        e.b[i] = (int)(16u * dx);
-                        e.c[i] = (int)(dy * (unsigned)o.x[p] - dx * (unsigned)o.y[p] - (unsigned)(((owns_bits >> i) & 1) ^ 1));
-                        e.iz[i] = o.iz[i];
+    }
+    if (VC && base + lane + NT < a.n) {
+        t_next = a.list ? a.list[base + lane + NT] : base + lane + NT;
+        tv_next = __ldg(&a.tris[t_next]);
+    }
+    for (;;) {
+        if (count < 32 && base < a.n) {
+            const int i = base + lane;
+            const int4 tv = tv_next;
+            uint4 e = e_next;
+            if (VC) {
+                if (i + NT < a.n) {
+                    e_next = make_uint4((uint32_t)a.vc[tv.x], (uint32_t)a.vc[tv.y], (uint32_t)a.vc[tv.z], (unsigned)t_next);
+                    if (i + 2 * NT < a.n) {
+                        t_next = a.list ? a.list[i + 2 * NT] : i + 2 * NT;
+                        tv_next = __ldg(&a.tris[t_next]);
                     }
-                    e.A = o.A;
-                    e.tri = t;
-                    e.uv0 = u0 | (v0 << 16);
-                    e.bw_bias = (u1 - u0 + 1) | ((~owns_bits & 7) << 16);
-                    TS[lane] = e;                  // whole-record store
+                }
+            } else if (i + NT < a.n) {
+                t_next = a.list ? a.list[i + NT] : i + NT;
+                tv_next = __ldg(&a.tris[t_next]);
+                e_next.w = (unsigned)t_next;
+            }
+            base += NT;
+            bool some = false;
+            if (i < a.n) {
+                if (VC) {
+                    const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
+                    const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
+                    const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
+                    some = __vmaxu2(pl, ph) == ph && (hi & 0xFFFFu) != 0xFFFFu;
+                } else {
+                    TriSetup o;
+                    some = load_triangle(cam, cam.verts, cam.P, tv, o) &&
+                           max(ceil16(min(o.x[0], min(o.x[1], o.x[2]))), a.tu0) <=
+                               min(floor16(max(o.x[0], max(o.x[1], o.x[2]))), a.tu1 - 1) &&
+                           max(ceil16(min(o.y[0], min(o.y[1], o.y[2]))), a.tv0) <=
+                               min(floor16(max(o.y[0], max(o.y[1], o.y[2]))), a.tv1 - 1);
                 }
             }
+            const unsigned bal = __ballot_sync(0xffffffffu, some);
+            if (some) TR[(head + count + __popc(bal & lt)) & (kRing - 1)] = e;
+            count += __popc(bal);
+            continue;
         }
-        // the larger boxes: their samples spread evenly over the lanes
-        if (__ballot_sync(0xffffffffu, area > 0) == 0u) continue;
-        int incl = area;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            int x = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += x;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        const bool last = count == 0;                   // only covered samples left
+        if (last && dcount == 0) break;
         __syncwarp();
-        for (int f0 = 0; f0 < total; f0 += 32) {
-            const int f = f0 + lane;
-            // the triangle j whose pixel range holds f: incl[j-1] <= f < incl[j]
-            int j = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                int v = __shfl_sync(0xffffffffu, incl, j + step - 1);
-                if (v <= f) j += step;
+        // ---- set-up of the 32 oldest, one per lane: sample state (x0, x1, K, tri,
+        // idx), per column (a0, a1) and, at the end of a row of bw, (r0, r1)
+        int x0, x1, K, tri, a0, a1, r0, r1, bw, left, items = 0, first, total;
+        unsigned idx;
+        {
+            const bool have = lane < count;
+            const uint4 e = TR[(head + lane) & (kRing - 1)];
+            tri = (int)e.w;
+            head = (head + 32) & (kRing - 1);
+            count = max(0, count - 32);
+            int x[3], y[3], u0, v0, bh;
+            if (VC) {
+                const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
+                const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
+                const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
+                u0 = (int)(pl & 0xFFFFu); v0 = (int)(pl >> 16);
+                bw = (int)(ph & 0xFFFFu) - u0 + 1; bh = (int)(ph >> 16) - v0 + 1;
+                x[0] = (int)(e.x & 0xFFFFu); x[1] = (int)(e.y & 0xFFFFu); x[2] = (int)(e.z & 0xFFFFu);
+                y[0] = (int)(e.x >> 16); y[1] = (int)(e.y >> 16); y[2] = (int)(e.z >> 16);
+            } else {
+                TriSetup o;
+                for (int k = 0; k < 3; ++k) o.x[k] = o.y[k] = 0;
+                if (have) load_triangle(cam, cam.verts, cam.P, __ldg(&a.tris[tri]), o);
+                for (int k = 0; k < 3; ++k) { x[k] = o.x[k]; y[k] = o.y[k]; }
+                u0 = max(ceil16(min(x[0], min(x[1], x[2]))), a.tu0);
+                v0 = max(ceil16(min(y[0], min(y[1], y[2]))), a.tv0);
+                bw = min(floor16(max(x[0], max(x[1], x[2]))), a.tu1 - 1) - u0 + 1;
+                bh = min(floor16(max(y[0], max(y[1], y[2]))), a.tv1 - 1) - v0 + 1;
             }
-            const int excl = __shfl_sync(0xffffffffu, incl, j > 0 ? j - 1 : 0);
-            if (f >= total) continue;
-            const TriStage e = TS[j];              // whole-record load
-            const int local = f - (j > 0 ? excl : 0);
-            const int bw = e.bw_bias & 0xFFFF;
-            const int dv = div_small(local, bw);
-            raster_staged<K32>(e, (e.uv0 & 0xFFFF) + (local - dv * bw), (e.uv0 >> 16) + dv, zbuf, tu0, tv0, tw, tcap,
-                               err);
+            // edge i runs from vertex i + 1 to vertex i + 2 (mod 3), all reversed when
+            // the area is negative (two-sided rendering)
+            int A = edge_fn(x[0], y[0], x[1], y[1], x[2], y[2]);
+            const int sg = A < 0 ? -1 : 1;
+            A = abs(A);
+            const int area = have && A != 0 ? bw * bh : 0;  // 0: nothing to do
+            const int dx0 = sg * (x[2] - x[1]), dy0 = sg * (y[2] - y[1]), dx1 = sg * (x[0] - x[2]), dy1 = sg * (y[0] - y[2]);
+            const int n0 = owns(dx0, dy0) ? 0 : 1, n1 = owns(dx1, dy1) ? 0 : 1;
+            K = A - n0 - n1 - (owns(sg * (x[1] - x[0]), sg * (y[1] - y[0])) ? 0 : 1);
+            a0 = -16 * dy0; a1 = -16 * dy1;
+            // edge values at the box's first sample, less the tie bias
+            x0 = (int)((unsigned)dx0 * (unsigned)(16 * v0 - y[1]) - (unsigned)dy0 * (unsigned)(16 * u0 - x[1]) - (unsigned)n0);
+            x1 = (int)((unsigned)dx1 * (unsigned)(16 * v0 - y[2]) - (unsigned)dy1 * (unsigned)(16 * u0 - x[2]) - (unsigned)n1);
+            idx = (unsigned)((v0 - kPix - a.tv0) * a.tw + (u0 - kPix - a.tu0)) | (unsigned)((n0 << 16) | (n1 << 17));
+            left = area <= kTinyBox ? area : 0;
+            r0 = 16 * dx0 - (bw - 1) * a0;
+            r1 = 16 * dx1 - (bw - 1) * a1;
+            // ---- the larger boxes: staged, or back to the queue
+            const unsigned big = __ballot_sync(0xffffffffu, area > kTinyBox);
+            first = total = 0;
+            if (big != 0u) {
+                const int rank = __popc(big & lt), n_big = __popc(big);
+                if (area > kTinyBox && rank >= kStaged) TR[(head + count + rank - kStaged) & (kRing - 1)] = e;
+                count += max(0, n_big - kStaged);
+                // thin: the triangle's area (A / 512 samples) is under a quarter of the box's
+                const bool thin = bw > 2 && (long long)A < 128ll * area;
+                items = area > kTinyBox && rank < kStaged ? (thin ? bh : area) : 0;
+                first = items;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int v = __shfl_up_sync(0xffffffffu, first, off);
+                    if (lane >= off) first += v;
+                }
+                total = __shfl_sync(0xffffffffu, first, 31);
+                first -= items;
+                if (items > 0)
+                    TS[rank] = TriStage{a0, a1, 16 * dx0, 16 * dx1, x0, x1, K, tri, idx | (thin ? 1u << 18 : 0u), bw,
+                                        __frcp_rn(__int2float_rn(bw)), first};
+                __syncwarp();
+            }
         }
-        __syncwarp();
+        int du = bw, begun = 0;                         // begun: staged triangles whose items began before f0
+        for (int f0 = 0;; f0 += 32) {
+            // ---- walk the lanes' samples
+            while (__ballot_sync(0xffffffffu, left > 0) != 0u || (last && dcount > 0)) {
+                // covered: every edge value, less its tie bias, is non-negative
+                const bool cov = left > 0 && (x0 | x1 | (int)((unsigned)K - (unsigned)x0 - (unsigned)x1)) >= 0;
+                const unsigned bal = __ballot_sync(0xffffffffu, cov);
+                if (cov) DQ[(dhead + dcount + __popc(bal & lt)) & (kRing - 1)] = DepthItem{x0, x1, tri, idx};
+                dcount += __popc(bal);
+                --left;
+                const bool wrap = --du == 0;            // on to the next row
+                x0 = (int)((unsigned)x0 + (unsigned)(wrap ? r0 : a0));
+                x1 = (int)((unsigned)x1 + (unsigned)(wrap ? r1 : a1));
+                idx += wrap ? (unsigned)(a.tw - (bw - 1)) : 1u;
+                if (wrap) du = bw;
+                if (dcount >= 32 || last) {
+                    const int n = min(dcount, 32);
+                    depth_flush<K32, VC>(a, cam, dhead, n, lane);
+                    dhead = (dhead + n) & (kRing - 1);
+                    dcount -= n;
+                }
+            }
+            if (f0 >= total) break;
+            // ---- the next 32 items: item f belongs to the last triangle begun at or before it
+            const unsigned rel = (unsigned)(first - f0);
+            const unsigned starts = __reduce_or_sync(0xffffffffu, items > 0 && rel < 32u ? 1u << rel : 0u);
+            begun += __popc(starts & (lt | (1u << lane)));
+            const TriStage s = TS[begun - 1];
+            begun = __shfl_sync(0xffffffffu, begun, 31);
+            const int f = f0 + lane, local = f - s.first;
+            int u, v = local;                           // the item's samples: `left` of row v from column u
+            x0 = s.t0; x1 = s.t1; K = s.K; tri = s.tri; a0 = s.a0; a1 = s.a1;
+            if (s.idx & (1u << 18)) {
+                x0 = (int)((unsigned)x0 + (unsigned)s.b0 * (unsigned)v);
+                x1 = (int)((unsigned)x1 + (unsigned)s.b1 * (unsigned)v);
+                // where the row crosses the edges: u < 2^16 and the quotient's relative
+                // error is below 2^-21, so the margin of 1/16 keeps every covered sample
+                float lo = 0.0f, hi = (float)(s.bw - 1);
+                const int xs[3] = {x0, x1, (int)((unsigned)K - (unsigned)x0 - (unsigned)x1)};
+                const int as[3] = {a0, a1, -a0 - a1};
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const float r = __fdividef(-__int2float_rn(xs[k]), __int2float_rn(as[k]));
+                    if (as[k] > 0) lo = fmaxf(lo, r - 0.0625f);
+                    else if (as[k] < 0) hi = fminf(hi, r + 0.0625f);
+                    else if (xs[k] < 0) hi = -1.0f;
+                }
+                u = __float2int_ru(fminf(lo, 65536.0f));
+                left = __float2int_rd(fmaxf(hi, -1.0f)) - u + 1;
+            } else {
+                v = __float2int_rz(__fmul_rn(__int2float_rn(local), s.rbw));
+                const int r = local - v * s.bw;
+                v += (r >= s.bw) - (r < 0);
+                u = local - v * s.bw;
+                left = 1;
+                x0 = (int)((unsigned)x0 + (unsigned)s.b0 * (unsigned)v);
+                x1 = (int)((unsigned)x1 + (unsigned)s.b1 * (unsigned)v);
+            }
+            if (f >= total) left = 0;
+            x0 = (int)((unsigned)x0 + (unsigned)a0 * (unsigned)u);
+            x1 = (int)((unsigned)x1 + (unsigned)a1 * (unsigned)u);
+            idx = (s.idx & 0x3FFFFu) + (unsigned)(v * a.tw + u);
+            du = INT_MAX;
+        }
     }
+}
+
+// raster_tile of mesh m (or of its triangles list[0 .. n_list)) at pose P.
+// probe_off and ring_off: byte offsets of the block's per-warp scratch and of its
+// warps' depth rings in shared memory.
+template <int NT, bool K32, bool VC>
+__device__ __forceinline__ void raster(const DevScene& sc, const DevMesh& m, const float* P,
+                                       const unsigned long long* vc, unsigned probe_off, unsigned ring_off, int tu0,
+                                       int tv0, int tu1, int tv1, int tw, int* err, const int* list = nullptr,
+                                       int n_list = 0)
+{
+    const unsigned warp = threadIdx.x >> 5;
+    const RasterArgs a = {m.tris, vc, list, list ? n_list : m.n_tris, tu0, tv0, tu1, tv1, tw,
+                          probe_off + warp * (unsigned)kWarpScratch,
+                          ring_off + warp * (unsigned)(kRing * sizeof(DepthItem)), err};
+    RasterCamera cam = {};
+    if (!VC) cam = {m.verts, P, sc.W, sc.H, sc.fx, sc.fy, sc.cx, sc.cy, sc.z_near};
+    raster_tile<NT, K32, VC>(a, cam);
 }
 
 // Tile bins of one hypothesis: the pixel box rbox is rasterised in tiles of tw
@@ -1377,10 +1557,9 @@ __device__ __forceinline__ uint32_t interp_colour(const DevMesh& m, const TriSet
     // integer arithmetic
     const float rA = __frcp_rn(__int2float_rn(o.A));
     uint32_t crgb = 0;
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-        const long long num = w0 * ((c0 >> (8 * ch)) & 255) + w1 * ((c1 >> (8 * ch)) & 255) +
-                              w2 * ((c2 >> (8 * ch)) & 255) + half;
+#pragma unroll 1
+    for (int ch = 0; ch < 24; ch += 8) {
+        const long long num = w0 * ((c0 >> ch) & 255) + w1 * ((c1 >> ch) & 255) + w2 * ((c2 >> ch) & 255) + half;
         // num < 2^41: its binary32 value from two 32-bit halves (the
         // estimate needs only relative accuracy, the correction makes it exact)
         const float numf = __fadd_rn(__fmul_rn(__int2float_rn((int)(num >> 16)), 65536.0f),
@@ -1388,7 +1567,7 @@ __device__ __forceinline__ uint32_t interp_colour(const DevMesh& m, const TriSet
         long long q = __float2int_rz(__fmul_rn(numf, rA));
         const long long r = num - q * o.A;
         q += (r >= o.A) - (r < 0);
-        crgb |= (uint32_t)q << (8 * ch);
+        crgb |= (uint32_t)q << ch;
     }
     return crgb;
 }
@@ -1451,30 +1630,26 @@ __device__ __forceinline__ bool in_admissible(const DevScene& sc, const Job& J, 
 
 // |I cap V| of plain scoring, counted in chunks of kJoChunk lattice pixels of
 // the whole admissible box taken from a shared counter (zero at the start of
-// the hypothesis).  It needs nothing rendered, so warps that finish the
-// raster early count chunks while the others still rasterise (`stop`: the
-// count of warps done with the raster; they stop once all are), and the
-// chunks left over are counted after the search.
+// the hypothesis).  It needs nothing rendered: a warp counts chunks once the
+// search leaves it idle, so the warps that finish early count most of them.
 constexpr int kJoChunk = 256;
 
-template <int NT>
-__device__ void jo_count_in(const DevScene& sc, const Job& J, const float* P, const int* vbox, int* counter,
-                            const int* stop, int& n_in)
+__device__ __forceinline__ void jo_count_in(const DevScene& sc, const Job& J, const float* P, const int* vbox,
+                                            int* counter, int& n_in)
 {
     const int s = sc.stride, lane = threadIdx.x & 31;
-    const int us0 = ((vbox[0] + s - 1) / s) * s, vs0 = ((vbox[1] + s - 1) / s) * s;
-    const int nu = us0 < vbox[2] ? (vbox[2] - 1 - us0) / s + 1 : 0;
-    const int nv = vs0 < vbox[3] ? (vbox[3] - 1 - vs0) / s + 1 : 0;
+    const int us0 = div_small(vbox[0] + s - 1, s) * s, vs0 = div_small(vbox[1] + s - 1, s) * s;
+    const int nu = us0 < vbox[2] ? div_small(vbox[2] - 1 - us0, s) + 1 : 0;
+    const int nv = vs0 < vbox[3] ? div_small(vbox[3] - 1 - vs0, s) + 1 : 0;
     const int npx = nu * nv;
     const float rr = __fmul_rn(J.m.vol_r, J.m.vol_r);
     for (;;) {
-        // one lane looks whether to stop and takes the chunk, so that the warp
-        // leaves the loop as one whatever the other warps do meanwhile
-        int c = INT_MAX / kJoChunk;
-        if (lane == 0 && !(stop && *reinterpret_cast<const volatile int*>(stop) >= NT / 32)) c = atomicAdd(counter, 1);
+        int c = 0;
+        if (lane == 0) c = atomicAdd(counter, 1);
         const int k0 = __shfl_sync(0xffffffffu, c, 0) * kJoChunk;
         if (k0 >= npx) break;
         const int k1 = min(k0 + kJoChunk, npx);
+#pragma unroll 1
         for (int k = k0 + lane; k < k1; k += 32) {
             const int kv = div_small(k, nu);
             const int pix = (vs0 + kv * s) * sc.W + us0 + (k - kv * nu) * s;
@@ -1488,7 +1663,7 @@ __device__ void jo_count_in(const DevScene& sc, const Job& J, const float* P, co
 // J_r is accumulated when count_jr; marks are set for nearest neighbours that
 // fall in rows [mv0, mv1) of the admissible box vbox.
 template <int NT, bool K32, bool VC, int MODE, bool BINS>
-__device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, const unsigned long long* vc,
+__device__ __forceinline__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, const unsigned long long* vc,
                             const int* rbox, const ScoreSmem& S, const int* vbox, int mv0, int mv1,
                             bool count_jr, int& jr_local, int& n_in, int& n_marked)
 {
@@ -1496,19 +1671,20 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
     const DevScene& sc = J.sc;
     const float rr = __fmul_rn(J.m.vol_r, J.m.vol_r);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    WarpProbe& WP = *reinterpret_cast<WarpProbe*>(reinterpret_cast<char*>(S.probe) + warp * kWarpScratch);
-    TriStage* TS = reinterpret_cast<TriStage*>(reinterpret_cast<char*>(S.stage) + warp * kWarpScratch);
+    WarpProbe& WP = *reinterpret_cast<WarpProbe*>(g_smem + a.probe_off + warp * (unsigned)kWarpScratch);
     const int s = sc.stride;
     const int rw = rbox[2] - rbox[0], rh = rbox[3] - rbox[1];
-    if (rw <= 0 || rh <= 0) return;
+    // (plain scoring goes through one empty tile, to count J_o's |I cap V|)
+    if (MODE != kModePlain && (rw <= 0 || rh <= 0)) return;
     const int cap_px = K32 ? a.zcap_words : a.zcap_words / 2;
-    const int tw = min(rw, cap_px);
-    const int th = max(1, cap_px / tw);
+    const int tw = max(1, min(rw, cap_px));
+    const int th = max(1, div_small(cap_px, tw));
     const uint32_t empty32 = 0xFFFFFFFFu;
     const int vw = vbox[2] - vbox[0];
-    uint32_t* zbuf = S.zbuf;
+    uint32_t* const zbuf = reinterpret_cast<uint32_t*>(g_smem);
+    uint32_t* const marks = reinterpret_cast<uint32_t*>(g_smem + a.marks_off);
     // a pixel box of several tiles: each tile's triangles binned first
-    const int n_tx = (rw + tw - 1) / tw, n_tiles = n_tx * ((rh + th - 1) / th);
+    const int n_tx = BINS ? (rw + tw - 1) / tw : 1, n_tiles = BINS ? n_tx * ((rh + th - 1) / th) : 1;
     const bool binned = BINS && VC && a.bin_cap > 0 && n_tiles > 1 && n_tiles <= kBinTiles;
     int* bins = binned ? reinterpret_cast<int*>(const_cast<unsigned long long*>(vc) + a.bin_off) : nullptr;
     if (binned) {
@@ -1518,28 +1694,21 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
         __syncthreads();
     }
     int tile = 0;
-    for (int tv0 = rbox[1]; tv0 < rbox[3]; tv0 += th) {
-        for (int tu0 = rbox[0]; tu0 < rbox[2]; tu0 += tw, ++tile) {
+    int tv0 = rbox[1];
+    do {
+        int tu0 = rbox[0];
+        do {
             const int tu1 = min(tu0 + tw, rbox[2]), tv1 = min(tv0 + th, rbox[3]);
             const int tpx = tw * (tv1 - tv0);
             const int words = K32 ? tpx : 2 * tpx;
+#pragma unroll 1
             for (int i = threadIdx.x; i < words; i += NT) zbuf[i] = empty32;
-            if (threadIdx.x == 0) {
-                *S.next_batch = 0;
-                *S.raster_done = 0;
-            }
+            if (threadIdx.x == 0) *S.next_batch = 0;
             __syncthreads();
-            if (BINS && binned && S.bin_cnt[tile] <= a.bin_cap)
-                raster_tile<NT, K32, VC, BINS>(sc, J.m, P, vc, TS, zbuf, tu0, tv0, tu1, tv1, tw, a.err,
-                                               bins + tile * a.bin_cap, S.bin_cnt[tile]);
-            else
-                raster_tile<NT, K32, VC>(sc, J.m, P, vc, TS, zbuf, tu0, tv0, tu1, tv1, tw, a.err);
-            if (MODE == kModePlain && count_jr) {
-                // the raster's early finishers count J_o's |I cap V| meanwhile
-                if (lane == 0) atomicAdd(S.raster_done, 1);
-                __syncwarp();
-                jo_count_in<NT>(sc, J, P, vbox, S.jo_next, S.raster_done, n_in);
-            }
+            // (the depth rings take the place of the kept-point queues, idle meanwhile)
+            const bool in_bin = BINS && binned && S.bin_cnt[tile] <= a.bin_cap;
+            raster<NT, K32, VC>(sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw, a.err,
+                                in_bin ? bins + tile * a.bin_cap : nullptr, in_bin ? S.bin_cnt[tile] : 0);
             __syncthreads();
             if (a.dump) {
                 for (int i = threadIdx.x; i < tpx; i += NT) {
@@ -1561,13 +1730,13 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
             // warp resolves a block (occluder test, colour, back-projection)
             // and appends its kept points to its own queue, which it searches
             // 32 at a time -- no block-wide barrier until the tile is done.
-            const int us0 = ((tu0 + s - 1) / s) * s, vs0 = ((tv0 + s - 1) / s) * s;
-            const int nu = us0 < tu1 ? (tu1 - 1 - us0) / s + 1 : 0;
-            const int nv = vs0 < tv1 ? (tv1 - 1 - vs0) / s + 1 : 0;
+            const int us0 = div_small(tu0 + s - 1, s) * s, vs0 = div_small(tv0 + s - 1, s) * s;
+            const int nu = us0 < tu1 ? div_small(tu1 - 1 - us0, s) + 1 : 0;
+            const int nv = vs0 < tv1 ? div_small(tv1 - 1 - vs0, s) + 1 : 0;
             const int nbx = (nu + 7) / 8, nby = (nv + 3) / 4;
             const int nblocks = nbx * nby;
-            KeptPoint* wq = S.kept + warp * kWarpQueue;
-            const MarkBand mband = {S.marks, vbox[0], vbox[2], mv0, mv1, vw, a.err};
+            KeptPoint* const wq = reinterpret_cast<KeptPoint*>(g_smem + a.kept_off) + warp * kWarpQueue;
+            const MarkBand mband = {marks, vbox[0], vbox[2], mv0, mv1, vw, a.err};
             __syncwarp();
             int wq_head = 0, wq_count = 0;
             for (;;) {
@@ -1628,7 +1797,7 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
                         }
                     }
                     const unsigned bal = __ballot_sync(0xffffffffu, kept);
-                    if (kept) wq[(wq_head + wq_count + __popc(bal & ((1u << lane) - 1u))) % kWarpQueue] = kp;
+                    if (kept) wq[(wq_head + wq_count + __popc(bal & ((1u << lane) - 1u))) & (kWarpQueue - 1)] = kp;
                     wq_count += __popc(bal);
                 }
                 // search a full batch, or what is left once the blocks run out
@@ -1637,8 +1806,8 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
                     const int nb = min(wq_count, 32);
                     const bool valid = lane < nb;
                     KeptPoint kq = {0.f, 0.f, 0.f, 0u};
-                    if (valid) kq = wq[(wq_head + lane) % kWarpQueue];
-                    wq_head = (wq_head + nb) % kWarpQueue;
+                    if (valid) kq = wq[(wq_head + lane) & (kWarpQueue - 1)];
+                    wq_head = (wq_head + nb) & (kWarpQueue - 1);
                     wq_count -= nb;
                     const uint32_t qpix = (EQ3 && valid) ? kq.pix : 0u;
                     const unsigned long long nn = probe_batch<EQ3, true>(sc, valid, kq.x, kq.y, kq.z, qpix, WP, lane, mband);
@@ -1670,7 +1839,7 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
                                 int bit = (pv - mv0) * vw + (pu - vbox[0]);
                                 if (PERCH_CHECKED((unsigned)bit < 32u * (unsigned)a.mark_words, a.err)) {
                                     const unsigned m = 1u << (bit & 31);
-                                    const unsigned was = atomicOr(&S.marks[bit >> 5], m);
+                                    const unsigned was = atomicOr(&marks[bit >> 5], m);
                                     if (MODE == kModePlain && !(was & m)) {
                                         // J_o's marked part: the first mark of a pixel of V
                                         const int npix = pv * sc.W + pu;
@@ -1684,11 +1853,36 @@ __device__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, co
                 }
                 if (!more) break;
             }
+            // J_o's |I cap V|, by the warps that finish the search first (all of it
+            // with the first tile)
+            if (MODE == kModePlain && count_jr) jo_count_in(sc, J, P, vbox, S.jo_next, n_in);
             __syncthreads();
             if (threadIdx.x == 0) *S.next_batch = 0;
             __syncthreads();
-        }
-    }
+            ++tile;
+            tu0 += tw;
+        } while (tu0 < rbox[2]);
+        tv0 += th;
+    } while (tv0 < rbox[3]);
+}
+
+// score_tiles without the vertex cache (images over 1023 pixels) or with 64-bit
+// keys (65,536 triangles or more, poses beyond 6.5 m): called, so that the
+// common case has the kernel's registers and instruction cache to itself.
+// Returns (J_r, |I cap V|, marked) of this thread.
+template <int NT, int MODE, bool BINS>
+__device__ __noinline__ int3 score_tiles_rare(const ScoreArgs& a, const float* P, const unsigned long long* vc,
+                                              const int* rbox, ScoreSmem S, const int* vbox, int mv0, int mv1,
+                                              bool count_jr, int k32)
+{
+    int3 r = make_int3(0, 0, 0);
+    if (vc)
+        score_tiles<NT, false, true, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+    else if (k32)
+        score_tiles<NT, true, false, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+    else
+        score_tiles<NT, false, false, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+    return r;
 }
 
 // jo_mode 1 with the colour check, after score_tiles has made every key of
@@ -1700,8 +1894,6 @@ __device__ __noinline__ void jo_colour_band(const ScoreArgs& a, const Job& J, co
                                             const unsigned long long* vc, const int* rbox, const ScoreSmem& S,
                                             const int* vbox, int mv0, int mv1)
 {
-    const int warp = threadIdx.x >> 5;
-    TriStage* TS = reinterpret_cast<TriStage*>(reinterpret_cast<char*>(S.stage) + warp * kWarpScratch);
     const int rw = rbox[2] - rbox[0], rh = rbox[3] - rbox[1];
     if (rw <= 0 || rh <= 0) return;
     const int cap_px = K32 ? a.zcap_words : a.zcap_words / 2;
@@ -1718,7 +1910,7 @@ __device__ __noinline__ void jo_colour_band(const ScoreArgs& a, const Job& J, co
             const int words = K32 ? tw * (tv1 - tv0) : 2 * tw * (tv1 - tv0);
             for (int i = threadIdx.x; i < words; i += NT) S.zbuf[i] = 0xFFFFFFFFu;
             __syncthreads();
-            raster_tile<NT, K32, VC>(J.sc, J.m, P, vc, TS, S.zbuf, tu0, tv0, tu1, tv1, tw, a.err);
+            raster<NT, K32, VC>(J.sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw, a.err);
             __syncthreads();
             jo_colour_pass<NT, K32, VC>(J, P, vc, S, tu0, tv0, tu1, tv1, tw, vbox, mv0, mv1);
             __syncthreads();
@@ -1739,19 +1931,20 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
     if (threadIdx.x == 0) *S.jo_next = 0;
     if (threadIdx.x < 4) S.vbounds[threadIdx.x] = threadIdx.x < 2 ? INT_MAX : INT_MIN;
     __syncthreads();
-    // the two boxes in two warps, in parallel with each other and with the
-    // other warps' share of the vertex pass
-    if (threadIdx.x == 0) {
-        float zmax;
-        project_box(sc, s_pose, J.m.lo, J.m.hi, J.roi[0], J.roi[1], J.roi[2], J.roi[3], s_rbox, &zmax);
-        *s_k32 = (J.m.n_tris <= 65535 && zmax < 6.5f) ? 1 : 0;
-    } else if (threadIdx.x == 32) {
-        if (J.label >= 0) {
-            s_vbox[0] = J.roi[0]; s_vbox[1] = J.roi[1]; s_vbox[2] = J.roi[2]; s_vbox[3] = J.roi[3];
-        } else {
-            float lo[3] = {-J.m.vol_r, -J.m.vol_r, 0.0f}, hi[3] = {J.m.vol_r, J.m.vol_r, J.m.vol_h};
-            float zv;
-            project_box(sc, s_pose, lo, hi, 0, 0, sc.W, sc.H, s_vbox, &zv);
+    // the two boxes by two warps, while the others begin the vertex pass
+    if (threadIdx.x < 64) {
+        const DevMesh& m = J.m;
+        const bool vol = threadIdx.x >= 32;
+        const PixelBox b = project_box(
+            make_float4(sc.fx, sc.fy, sc.cx, sc.cy), s_pose,
+            vol ? make_float3(-m.vol_r, -m.vol_r, 0.0f) : make_float3(m.lo[0], m.lo[1], m.lo[2]),
+            vol ? make_float3(m.vol_r, m.vol_r, m.vol_h) : make_float3(m.hi[0], m.hi[1], m.hi[2]),
+            vol ? make_int4(0, 0, sc.W, sc.H) : make_int4(J.roi[0], J.roi[1], J.roi[2], J.roi[3]));
+        if ((threadIdx.x & 31) == 0) {
+            int* const out = vol ? s_vbox : s_rbox;
+            out[0] = b.box.x; out[1] = b.box.y; out[2] = b.box.z; out[3] = b.box.w;
+            if (!vol) *s_k32 = (m.n_tris <= 65535 && b.zmax < 6.5f) ? 1 : 0;
+            else if (J.label >= 0) for (int i = 0; i < 4; ++i) out[i] = J.roi[i];
         }
     }
     const bool use_vc = vc != nullptr;
@@ -1761,17 +1954,16 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
     // (with the vertex cache) to the samples between the kept vertices'
     // smallest and largest snapped coordinates -- every covered sample lies
     // in its triangle's vertex box, so nothing outside can be covered.
-    int rb[4] = {s_rbox[0], s_rbox[1], s_rbox[2], s_rbox[3]};
-    if (use_vc) {
+    if (threadIdx.x == 0 && use_vc) {
         const int* vb = S.vbounds;
         if (vb[0] > vb[2]) {
-            rb[2] = rb[0];
-            rb[3] = rb[1];
+            s_rbox[2] = s_rbox[0];
+            s_rbox[3] = s_rbox[1];
         } else {
-            rb[0] = max(rb[0], ceil16(vb[0]));
-            rb[1] = max(rb[1], ceil16(vb[1]));
-            rb[2] = max(rb[0], min(rb[2], floor16(vb[2]) + 1));
-            rb[3] = max(rb[1], min(rb[3], floor16(vb[3]) + 1));
+            s_rbox[0] = max(s_rbox[0], ceil16(vb[0]));
+            s_rbox[1] = max(s_rbox[1], ceil16(vb[1]));
+            s_rbox[2] = max(s_rbox[0], min(s_rbox[2], floor16(vb[2]) + 1));
+            s_rbox[3] = max(s_rbox[1], min(s_rbox[3], floor16(vb[3]) + 1));
         }
     }
 
@@ -1780,39 +1972,38 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
     // render + search (J_r counted once).
     constexpr bool jo1 = MODE == kModeEq3;
     const int vw = s_vbox[2] - s_vbox[0], vh = s_vbox[3] - s_vbox[1];
-    const int band_rows = vw > 0 ? max(1, (jo1 ? a.mark_words / 2 : 32 * a.mark_words) / vw) : 1;
-    const int n_bands = vh > 0 ? (vh + band_rows - 1) / band_rows : 1;
+    const int band_rows = vw > 0 ? max(1, div_small(jo1 ? a.mark_words / 2 : 32 * a.mark_words, vw)) : 1;
+    const int n_bands = vh > 0 ? div_small(vh + band_rows - 1, band_rows) : 1;
     int jr = 0, n_in = 0, n_marked = 0;
     const int s = sc.stride;
     const float* P = s_pose;
     const float rr = __fmul_rn(J.m.vol_r, J.m.vol_r);
+#pragma unroll 1
     for (int band = 0; band < n_bands; ++band) {
         const int mv0 = s_vbox[1] + band * band_rows;
         const int mv1 = min(mv0 + band_rows, s_vbox[3]);
         const int mwords = jo1 ? 2 * vw * max(0, mv1 - mv0) : (vw * max(0, mv1 - mv0) + 31) / 32;
         const uint32_t mfill = jo1 ? 0xFFFFFFFFu : 0u;     // empty keys / clear bits
+#pragma unroll 1
         for (int i = threadIdx.x; i < mwords; i += NT) S.marks[i] = mfill;
         __syncthreads();
-        if (*s_k32) {
-            if (use_vc) score_tiles<NT, true, true, MODE, BINS>(a, J, P, vc, rb, S, s_vbox, mv0, mv1, band == 0, jr,
-                                                               n_in, n_marked);
-            else score_tiles<NT, true, false, MODE, BINS>(a, J, P, vc, rb, S, s_vbox, mv0, mv1, band == 0, jr,
-                                                               n_in, n_marked);
+        if (*s_k32 && use_vc) {
+            score_tiles<NT, true, true, MODE, BINS>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, jr, n_in, n_marked);
         } else {
-            if (use_vc) score_tiles<NT, false, true, MODE, BINS>(a, J, P, vc, rb, S, s_vbox, mv0, mv1, band == 0, jr,
-                                                               n_in, n_marked);
-            else score_tiles<NT, false, false, MODE, BINS>(a, J, P, vc, rb, S, s_vbox, mv0, mv1, band == 0, jr,
-                                                               n_in, n_marked);
+            const int3 r = score_tiles_rare<NT, MODE, BINS>(a, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, *s_k32);
+            jr += r.x;
+            n_in += r.y;
+            n_marked += r.z;
         }
         __syncthreads();
         if (jo1 && sc.color_check) {
             // Eq. 4 from the observed side, once the band's keys are final
             if (*s_k32) {
-                if (use_vc) jo_colour_band<NT, true, true>(a, J, P, vc, rb, S, s_vbox, mv0, mv1);
-                else jo_colour_band<NT, true, false>(a, J, P, vc, rb, S, s_vbox, mv0, mv1);
+                if (use_vc) jo_colour_band<NT, true, true>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1);
+                else jo_colour_band<NT, true, false>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1);
             } else {
-                if (use_vc) jo_colour_band<NT, false, true>(a, J, P, vc, rb, S, s_vbox, mv0, mv1);
-                else jo_colour_band<NT, false, false>(a, J, P, vc, rb, S, s_vbox, mv0, mv1);
+                if (use_vc) jo_colour_band<NT, false, true>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1);
+                else jo_colour_band<NT, false, false>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1);
             }
         }
         // plain scoring: J_o's marked part was counted as the marks were set
@@ -1820,9 +2011,9 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
         // |I cap V| is counted by jo_count_in
         if (MODE == kModePlain) continue;
         // ---- J_o over the admissible set V(h), rows [mv0, mv1)
-        const int us0 = ((s_vbox[0] + s - 1) / s) * s, vs0 = ((mv0 + s - 1) / s) * s;
-        const int nu = us0 < s_vbox[2] ? (s_vbox[2] - 1 - us0) / s + 1 : 0;
-        const int nv = vs0 < mv1 ? (mv1 - 1 - vs0) / s + 1 : 0;
+        const int us0 = div_small(s_vbox[0] + s - 1, s) * s, vs0 = div_small(mv0 + s - 1, s) * s;
+        const int nu = us0 < s_vbox[2] ? div_small(s_vbox[2] - 1 - us0, s) + 1 : 0;
+        const int nv = vs0 < mv1 ? div_small(mv1 - 1 - vs0, s) + 1 : 0;
         // pixel k = (row k / nu, column k % nu), the row and column carried
         // from one k to the next (k advances by NT) instead of divided out
         int kr = nu > 0 ? div_small(threadIdx.x, nu) : 0, kc = threadIdx.x - kr * nu;
@@ -1863,8 +2054,6 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
         }
         __syncthreads();
     }
-    // the chunks of |I cap V| the raster's early finishers did not count
-    if (MODE == kModePlain) jo_count_in<NT>(sc, J, P, s_vbox, S.jo_next, nullptr, n_in);
     // ---- warp-shuffle reduction of (J_r, |I cap V|, marked)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1946,29 +2135,27 @@ __device__ int claim_vslot(unsigned* mask, int nslots)
 // Monotone Scene Generation tree from the state in job.tree.  At most 64
 // registers per thread (128 and 256 threads): four 256-thread blocks, 32 warps,
 // fit an SM when the block's shared memory allows (the default launch shape),
-// which hides latency better than three blocks of 80 registers.
+// which hides latency better than three blocks of 80 registers (36.6 against
+// 39.9 ms for three 640x480 objects x 29,584 poses).  The Eq. 3 scorer, which
+// holds more, would run from spilled values: 80 registers (2.44 against 2.84 ms
+// for two objects x 2,527 poses at 517x389).
 template <int NT, int MODE, bool BINS>
-__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 1024 / NT) k_score(const __grid_constant__ ScoreArgs a)
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : (MODE == kModeEq3 ? 768 : 1024) / NT) k_score(const __grid_constant__ ScoreArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char* const smem = g_smem;
     __shared__ float s_pose[12];
     __shared__ int s_rbox[4], s_vbox[4], s_k32, s_next, s_slot, s_refused, s_bin_cnt[kBinTiles], s_jo_next,
-        s_raster_done, s_vbounds[4];
+        s_vbounds[4];
     __shared__ long long s_h;
     __shared__ int s_red[3][NT / 32];
 
-    SmemLayout L = smem_layout(a.zcap_words, a.mark_words, NT);
     ScoreSmem S;
     S.zbuf = reinterpret_cast<uint32_t*>(smem);
-    S.marks = reinterpret_cast<uint32_t*>(smem + L.marks);
-    S.kept = reinterpret_cast<KeptPoint*>(smem + L.kept);
-    S.probe = reinterpret_cast<WarpProbe*>(smem + L.probe);
-    S.stage = reinterpret_cast<TriStage*>(smem + L.probe);
+    S.marks = reinterpret_cast<uint32_t*>(smem + a.marks_off);
     S.next_batch = &s_next;
     S.refused = &s_refused;
     S.bin_cnt = s_bin_cnt;
     S.jo_next = &s_jo_next;
-    S.raster_done = &s_raster_done;
     S.vbounds = s_vbounds;
     if (threadIdx.x == 0) s_slot = a.vcache ? claim_vslot(a.vmask, a.vslots) : -1;
     __syncthreads();
@@ -2009,9 +2196,14 @@ static int score_grid_nt(size_t smem)
 template <int NT>
 static int score_grid_all(size_t smem)
 {
-    // the specialisations share the vertex-cache pool: size for the smallest
-    return min(min(score_grid_nt<NT, kModePlain, false>(smem), score_grid_nt<NT, kModePlain, true>(smem)),
-               min(score_grid_nt<NT, kModeTree, false>(smem), score_grid_nt<NT, kModeEq3, false>(smem)));
+    // the specialisations share one grid and one vertex-cache pool: sized for the
+    // one with most resident blocks (of another, the blocks past its own share
+    // start as others end and find the counter spent)
+    const int g[4] = {score_grid_nt<NT, kModePlain, false>(smem), score_grid_nt<NT, kModePlain, true>(smem),
+                      score_grid_nt<NT, kModeTree, false>(smem), score_grid_nt<NT, kModeEq3, false>(smem)};
+    int most = g[0];
+    for (int k = 1; k < 4; ++k) most = g[k] < 0 || most < 0 ? -1 : max(most, g[k]);
+    return most;
 }
 
 int score_grid(const ScoreConfig& cfg, int mark_words)
@@ -2022,6 +2214,17 @@ int score_grid(const ScoreConfig& cfg, int mark_words)
     case 512: return score_grid_all<512>(smem);
     default: return score_grid_all<256>(smem);
     }
+}
+
+// a with the places of the block's shared-memory regions, which the kernel reads
+// from the parameter bank instead of holding them in registers.
+static ScoreArgs with_layout(ScoreArgs a, int threads)
+{
+    const SmemLayout L = smem_layout(a.zcap_words, a.mark_words, threads);
+    a.marks_off = (unsigned)L.marks;
+    a.kept_off = (unsigned)L.kept;
+    a.probe_off = (unsigned)L.probe;
+    return a;
 }
 
 // The kernel specialisation a launch runs on (tile bins: plain scoring only;
@@ -2043,7 +2246,7 @@ static cudaError_t launch_score_nt(const ScoreArgs& a, const ScoreConfig& cfg, i
     const void* fn = score_kernel<NT>(a);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    ScoreArgs copy = a;
+    ScoreArgs copy = with_layout(a, NT);
     void* args[] = {&copy};
     return cudaLaunchKernel(fn, dim3(g), dim3(NT), args, smem, s);
 }
@@ -2057,7 +2260,7 @@ static cudaError_t add_score_node_nt(cudaGraph_t g, const cudaGraphNode_t* deps,
     const void* fn = score_kernel<NT>(a);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    ScoreArgs copy = a;
+    ScoreArgs copy = with_layout(a, NT);
     void* args[] = {&copy};
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void*>(fn);
@@ -2346,11 +2549,9 @@ __device__ bool gicp_update(double* R, double* t, const double* xi, float stop_r
 // the number of source points (entries past cap are not written).
 template <int NT, bool K32, bool VC>
 __device__ void gicp_source(const GicpArgs& a, const Job& J, const float* P, const unsigned long long* vc,
-                            const int* rbox, uint32_t* zbuf, char* probe, float4* src, int* count)
+                            const int* rbox, uint32_t* zbuf, unsigned probe_off, float4* src, int* count)
 {
     const DevScene& sc = J.sc;
-    const int warp = threadIdx.x >> 5;
-    TriStage* TS = reinterpret_cast<TriStage*>(probe + warp * kWarpScratch);
     const int s = sc.stride;
     const int rw = rbox[2] - rbox[0], rh = rbox[3] - rbox[1];
     if (rw <= 0 || rh <= 0) return;
@@ -2363,7 +2564,8 @@ __device__ void gicp_source(const GicpArgs& a, const Job& J, const float* P, con
             const int words = K32 ? tw * (tv1 - tv0) : 2 * tw * (tv1 - tv0);
             for (int i = threadIdx.x; i < words; i += NT) zbuf[i] = 0xFFFFFFFFu;
             __syncthreads();
-            raster_tile<NT, K32, VC>(sc, J.m, P, vc, TS, zbuf, tu0, tv0, tu1, tv1, tw, a.err);
+            raster<NT, K32, VC>(sc, J.m, P, vc, probe_off, probe_off + (unsigned)kWarpScratch * (NT / 32), tu0, tv0,
+                                tu1, tv1, tw, a.err);
             __syncthreads();
             const int us0 = ((tu0 + s - 1) / s) * s, vs0 = ((tv0 + s - 1) / s) * s;
             const int nu = us0 < tu1 ? (tu1 - 1 - us0) / s + 1 : 0;
@@ -2410,7 +2612,7 @@ __host__ __device__ inline size_t gicp_probe_offset(int zcap_words)
 template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ GicpArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char* const smem = g_smem;
     __shared__ float s_pose[12], s_Rf[9], s_tf[3];
     __shared__ double s_R[9], s_t[3];
     __shared__ unsigned long long s_sum[kGicpTerms];
@@ -2420,7 +2622,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ G
     const Job& J = a.job;
     const DevScene& sc = J.sc;
     uint32_t* zbuf = reinterpret_cast<uint32_t*>(smem);
-    char* probe = reinterpret_cast<char*>(smem) + gicp_probe_offset(a.zcap_words);
+    const unsigned probe_off = (unsigned)gicp_probe_offset(a.zcap_words);
+    char* probe = reinterpret_cast<char*>(smem) + probe_off;
     WarpProbe& WP = *reinterpret_cast<WarpProbe*>(probe + warp * kWarpScratch);
     if (threadIdx.x == 0) {
         s_slot = claim_vslot(a.smask, a.slots);
@@ -2439,19 +2642,24 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ G
         if (threadIdx.x < 12) s_pose[threadIdx.x] = J.poses[h * 12 + threadIdx.x];
         if (threadIdx.x == 0) s_nsrc = 0;
         __syncthreads();
-        if (threadIdx.x == 0) {
-            float zmax;
-            project_box(sc, s_pose, J.m.lo, J.m.hi, J.roi[0], J.roi[1], J.roi[2], J.roi[3], s_rbox, &zmax);
-            s_k32 = (J.m.n_tris <= 65535 && zmax < 6.5f) ? 1 : 0;
+        if (threadIdx.x < 32) {
+            const PixelBox b = project_box(make_float4(sc.fx, sc.fy, sc.cx, sc.cy), s_pose,
+                                           make_float3(J.m.lo[0], J.m.lo[1], J.m.lo[2]),
+                                           make_float3(J.m.hi[0], J.m.hi[1], J.m.hi[2]),
+                                           make_int4(J.roi[0], J.roi[1], J.roi[2], J.roi[3]));
+            if (lane == 0) {
+                s_rbox[0] = b.box.x; s_rbox[1] = b.box.y; s_rbox[2] = b.box.z; s_rbox[3] = b.box.w;
+                s_k32 = (J.m.n_tris <= 65535 && b.zmax < 6.5f) ? 1 : 0;
+            }
         }
         if (vc) vertex_pass(sc, J.m, s_pose, const_cast<unsigned long long*>(vc), NT);
         __syncthreads();
         if (s_k32) {
-            if (vc) gicp_source<NT, true, true>(a, J, s_pose, vc, s_rbox, zbuf, probe, src, &s_nsrc);
-            else gicp_source<NT, true, false>(a, J, s_pose, vc, s_rbox, zbuf, probe, src, &s_nsrc);
+            if (vc) gicp_source<NT, true, true>(a, J, s_pose, vc, s_rbox, zbuf, probe_off, src, &s_nsrc);
+            else gicp_source<NT, true, false>(a, J, s_pose, vc, s_rbox, zbuf, probe_off, src, &s_nsrc);
         } else {
-            if (vc) gicp_source<NT, false, true>(a, J, s_pose, vc, s_rbox, zbuf, probe, src, &s_nsrc);
-            else gicp_source<NT, false, false>(a, J, s_pose, vc, s_rbox, zbuf, probe, src, &s_nsrc);
+            if (vc) gicp_source<NT, false, true>(a, J, s_pose, vc, s_rbox, zbuf, probe_off, src, &s_nsrc);
+            else gicp_source<NT, false, false>(a, J, s_pose, vc, s_rbox, zbuf, probe_off, src, &s_nsrc);
         }
         const int nsrc = s_nsrc;
         if (nsrc > a.src_cap) {
@@ -2555,7 +2763,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ G
 
 size_t gicp_smem_bytes(int zcap_words)
 {
-    return gicp_probe_offset(zcap_words) + kWarpScratch * (kGicpThreads / 32);
+    return gicp_probe_offset(zcap_words) + (kWarpScratch + sizeof(DepthItem) * kRing) * (kGicpThreads / 32);
 }
 
 int gicp_grid(int zcap_words)
