@@ -2306,11 +2306,14 @@ cudaError_t launch_score(const ScoreArgs& a, const ScoreConfig& cfg, int grid, c
 // within delta (the radius search of the scorer), contributes 28 binary32
 // terms (the 6x6 normal matrix's upper triangle, the gradient and r^T M r)
 // that are rounded to multiples of 2^-24 and summed exactly in int64, and
-// thread 0 solves the system in binary64 and updates the increment.  The
+// warp 0 solves the system in binary64 and updates the increment.  The
 // fixed-point sums make the result independent of the summation order.
 
 constexpr int kGicpTerms = 28;
-constexpr int kGicpThreads = 128;   // four blocks per SM: source clouds are small
+// Three blocks of 256 threads (80 registers) per SM: 24 warps.  With the warp-wide
+// solve: 26.8 ms for 20,480 refinements, against 32.0 ms for four blocks of 128
+// threads (128 registers, 16 warps) and 29.8 ms for five (96 registers).
+constexpr int kGicpThreads = 256;
 constexpr float kGicpScale = 16777216.0f;    // 2^24
 constexpr float kGicpLimit = 1048576.0f;     // a correspondence with a larger |term| is skipped
 
@@ -2461,63 +2464,79 @@ __device__ __forceinline__ bool gicp_terms(const float* Rf, float3 p, float4 na,
     return ok;
 }
 
-// rint(v) as a 64-bit integer for |v| < 2^46 without a 64-bit conversion:
-// below 2^31 a 32-bit round to nearest even; above, v is already an integer
-// (its ulp is at least 2^8) and splits exactly as 2^16 h + l, h = trunc(v /
-// 2^16) (the scaling is exact) and l = v - 2^16 h (exact: a multiple of 2^8
-// below 2^16 in magnitude).
-__device__ __forceinline__ long long rint_to_ll(float v)
+// rint(2^24 term) of each lane, summed over the warp: hi 2^22 + lo, |term| < 2^20.
+// Adding 1.5 x 2^23 rounds a binary32 value below 2^22 to an integer, ties to
+// even, and leaves it in the low bits: first 4 term (the multiples of 2^22, any
+// rounding will do), then the exact remainder, whose ties fall as the whole's
+// because 2^22 is even.  The biased bits of 32 lanes wrap, and the wrapped sum
+// less 32 biases is each sum exactly (|sum| < 2^27).  Two warp-wide integer
+// additions in place of five 64-bit shuffles, and no conversion instructions.
+__device__ __forceinline__ void warp_fixed_sum(float term, int& hi, int& lo)
 {
-    if (fabsf(v) < 2147483648.0f) return (long long)__float2int_rn(v);
-    const float h = truncf(__fmul_rn(v, 1.0f / 65536.0f));
-    const float l = __fsub_rn(v, __fmul_rn(h, 65536.0f));
-    return (long long)__float2int_rz(h) * 65536ll + (long long)__float2int_rz(l);
+    const float magic = 12582912.0f;             // 0x4B400000
+    const float t = __fmaf_rn(term, 4.0f, magic);
+    const float rest = __fmaf_rn(-__fsub_rn(t, magic), 4194304.0f, __fmul_rn(term, kGicpScale));
+    const unsigned h = __reduce_add_sync(0xffffffffu, __float_as_uint(t));
+    const unsigned l = __reduce_add_sync(0xffffffffu, __float_as_uint(__fadd_rn(rest, magic)));
+    hi = (int)(h - 32u * 0x4B400000u);
+    lo = (int)(l - 32u * 0x4B400000u);
 }
 
-// H xi = -g from the fixed-point sums, by Cholesky in binary64 (one thread).
-__device__ bool gicp_solve(const unsigned long long* S, double* xi)
+// H xi = -g from the fixed-point sums, by Cholesky in binary64, by one warp.
+// Lane k < 21 holds element (column c, row r >= c) of the lower triangle in the
+// sums' order, lane 21 + c the right-hand side as a row 6; column q is finished
+// (pivot, quotients) and subtracted from the columns after it, so every element
+// sees its subtractions in the order of q, as a row-by-row evaluation does, and
+// the result is that evaluation's to the bit.  The back substitution subtracts
+// in rising order too, which leaves it serial; all lanes do it.  One thread
+// alone took a sixth of a step: binary64 quotients and roots are long chains,
+// and here 12 of them follow one another instead of 33.
+__constant__ unsigned char c_gicp_col[27] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 2, 2, 2, 2, 3, 3, 3, 4, 4, 5, 0, 1, 2, 3, 4, 5};
+__constant__ unsigned char c_gicp_row[27] = {0, 1, 2, 3, 4, 5, 1, 2, 3, 4, 5, 2, 3, 4, 5, 3, 4, 5, 4, 5, 5, 6, 6, 6, 6, 6, 6};
+
+__host__ __device__ constexpr int gicp_lane(int c, int r)
 {
-    double H[6][6], g[6], L[6][6], y[6];
-    int k = 0;
-    for (int i = 0; i < 6; ++i)
-        for (int j = i; j < 6; ++j) {
-            H[i][j] = __ddiv_rn(__ll2double_rn((long long)S[k++]), 16777216.0);
-            H[j][i] = H[i][j];
-        }
-    for (int i = 0; i < 6; ++i) g[i] = __ddiv_rn(__ll2double_rn((long long)S[k++]), 16777216.0);
-    for (int j = 0; j < 6; ++j) {
-        double s = H[j][j];
-        for (int q = 0; q < j; ++q) s = __dsub_rn(s, __dmul_rn(L[j][q], L[j][q]));
-        if (!(s > 0.0)) return false;
-        L[j][j] = __dsqrt_rn(s);
-        for (int i = j + 1; i < 6; ++i) {
-            double t = H[i][j];
-            for (int q = 0; q < j; ++q) t = __dsub_rn(t, __dmul_rn(L[i][q], L[j][q]));
-            L[i][j] = __ddiv_rn(t, L[j][j]);
-        }
+    return r == 6 ? 21 + c : 6 * c - c * (c - 1) / 2 + r - c;
+}
+
+__device__ __forceinline__ bool gicp_solve(const unsigned long long* S, int lane, double* xi)
+{
+    const int k = min(lane, 26), c = c_gicp_col[k], r = c_gicp_row[k];
+    double t = __dmul_rn(__ll2double_rn((long long)S[k]), 1.0 / 16777216.0);     // exact scaling
+    if (r == 6) t = -t;
+#pragma unroll 1
+    for (int q = 0; q < 6; ++q) {
+        const double p = __shfl_sync(0xffffffffu, t, gicp_lane(q, q));
+        if (!(p > 0.0)) return false;
+        const double d = __dsqrt_rn(p);
+        if (c == q) t = r == q ? d : __ddiv_rn(t, d);
+        const double lr = __shfl_sync(0xffffffffu, t, gicp_lane(q, max(r, q)));
+        const double lc = __shfl_sync(0xffffffffu, t, gicp_lane(q, max(c, q)));
+        if (c > q) t = __dsub_rn(t, __dmul_rn(lr, lc));
     }
-    for (int i = 0; i < 6; ++i) {
-        double t = -g[i];
-        for (int q = 0; q < i; ++q) t = __dsub_rn(t, __dmul_rn(L[i][q], y[q]));
-        y[i] = __ddiv_rn(t, L[i][i]);
-    }
+#pragma unroll
     for (int i = 5; i >= 0; --i) {
-        double t = y[i];
-        for (int q = i + 1; q < 6; ++q) t = __dsub_rn(t, __dmul_rn(L[q][i], xi[q]));
-        xi[i] = __ddiv_rn(t, L[i][i]);
+        double x = __shfl_sync(0xffffffffu, t, gicp_lane(i, 6));
+#pragma unroll
+        for (int q = i + 1; q < 6; ++q) x = __dsub_rn(x, __dmul_rn(__shfl_sync(0xffffffffu, t, gicp_lane(i, q)), xi[q]));
+        xi[i] = __ddiv_rn(x, __shfl_sync(0xffffffffu, t, gicp_lane(i, i)));
     }
     return true;
 }
 
 // Apply the step xi to the increment (R, t): R <- dR R, t <- dR t + v, with
-// dR the rotation of the quaternion (1, w/2) normalised.  True when the step
-// is below the stopping thresholds.
-__device__ bool gicp_update(double* R, double* t, const double* xi, float stop_rot, float stop_trans)
+// dR the rotation of the quaternion (1, w/2) normalised; by one warp, lane 3 i +
+// j on R[i][j] and lane 9 + i on t[i].  True when the step is below the
+// stopping thresholds.
+__device__ __forceinline__ bool gicp_update(double* R, double* t, const double* xi, float stop_rot, float stop_trans,
+                                            int lane)
 {
     const double hx = __dmul_rn(xi[0], 0.5), hy = __dmul_rn(xi[1], 0.5), hz = __dmul_rn(xi[2], 0.5);
     const double nrm = __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(1.0, __dmul_rn(hx, hx)), __dmul_rn(hy, hy)),
                                             __dmul_rn(hz, hz)));
-    const double qw = __ddiv_rn(1.0, nrm), qx = __ddiv_rn(hx, nrm), qy = __ddiv_rn(hy, nrm), qz = __ddiv_rn(hz, nrm);
+    const double qk = __ddiv_rn(lane == 0 ? 1.0 : lane == 1 ? hx : lane == 2 ? hy : hz, nrm);
+    const double qw = __shfl_sync(0xffffffffu, qk, 0), qx = __shfl_sync(0xffffffffu, qk, 1);
+    const double qy = __shfl_sync(0xffffffffu, qk, 2), qz = __shfl_sync(0xffffffffu, qk, 3);
     double d[9];
     d[0] = __dsub_rn(1.0, __dmul_rn(2.0, __dadd_rn(__dmul_rn(qy, qy), __dmul_rn(qz, qz))));
     d[1] = __dmul_rn(2.0, __dsub_rn(__dmul_rn(qx, qy), __dmul_rn(qw, qz)));
@@ -2528,16 +2547,17 @@ __device__ bool gicp_update(double* R, double* t, const double* xi, float stop_r
     d[6] = __dmul_rn(2.0, __dsub_rn(__dmul_rn(qx, qz), __dmul_rn(qw, qy)));
     d[7] = __dmul_rn(2.0, __dadd_rn(__dmul_rn(qy, qz), __dmul_rn(qw, qx)));
     d[8] = __dsub_rn(1.0, __dmul_rn(2.0, __dadd_rn(__dmul_rn(qx, qx), __dmul_rn(qy, qy))));
-    double R2[9], t2[3];
-    for (int i = 0; i < 3; ++i) {
-        for (int j = 0; j < 3; ++j)
-            R2[3 * i + j] = __dadd_rn(__dadd_rn(__dmul_rn(d[3 * i], R[j]), __dmul_rn(d[3 * i + 1], R[3 + j])),
-                                      __dmul_rn(d[3 * i + 2], R[6 + j]));
-        t2[i] = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[3 * i], t[0]), __dmul_rn(d[3 * i + 1], t[1])),
-                                    __dmul_rn(d[3 * i + 2], t[2])), xi[3 + i]);
-    }
-    for (int i = 0; i < 9; ++i) R[i] = R2[i];
-    for (int i = 0; i < 3; ++i) t[i] = t2[i];
+    const int i = lane < 9 ? lane / 3 : min(lane - 9, 2), j = lane % 3;
+    const double d0 = i == 0 ? d[0] : i == 1 ? d[3] : d[6], d1 = i == 0 ? d[1] : i == 1 ? d[4] : d[7];
+    const double d2 = i == 0 ? d[2] : i == 1 ? d[5] : d[8];
+    const double* const col = lane < 9 ? R + j : t;
+    const int pitch = lane < 9 ? 3 : 1;
+    double x = __dadd_rn(__dadd_rn(__dmul_rn(d0, col[0]), __dmul_rn(d1, col[pitch])), __dmul_rn(d2, col[2 * pitch]));
+    if (lane >= 9) x = __dadd_rn(x, i == 0 ? xi[3] : i == 1 ? xi[4] : xi[5]);
+    __syncwarp();
+    if (lane < 9) R[lane] = x;
+    else if (lane < 12) t[i] = x;
+    __syncwarp();
     const double sr = (double)stop_rot, st = (double)stop_trans;
     const double w2 = __dadd_rn(__dadd_rn(__dmul_rn(xi[0], xi[0]), __dmul_rn(xi[1], xi[1])), __dmul_rn(xi[2], xi[2]));
     const double v2 = __dadd_rn(__dadd_rn(__dmul_rn(xi[3], xi[3]), __dmul_rn(xi[4], xi[4])), __dmul_rn(xi[5], xi[5]));
@@ -2610,7 +2630,7 @@ __host__ __device__ inline size_t gicp_probe_offset(int zcap_words)
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ GicpArgs a)
+__global__ void __launch_bounds__(NT, 768 / NT) k_gicp(const __grid_constant__ GicpArgs a)
 {
     unsigned char* const smem = g_smem;
     __shared__ float s_pose[12], s_Rf[9], s_tf[3];
@@ -2697,6 +2717,8 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ G
                 const unsigned long long nn = probe_batch<false, false>(sc, valid, p.x, p.y, p.z, 0u, WP, lane, nomark);
                 bool ok = valid && nn != kEmptyKey;
                 float terms[kGicpTerms];
+#pragma unroll
+                for (int j = 0; j < kGicpTerms; ++j) terms[j] = 0.0f;
                 if (ok) {
                     const uint32_t pw = (uint32_t)nn;
                     const int pu = (int)(pw & 0xFFFFu), pv = (int)(pw >> 16);
@@ -2709,26 +2731,29 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_gicp(const __grid_constant__ G
                 if (bal) {
 #pragma unroll
                     for (int j = 0; j < kGicpTerms; ++j) {
-                        long long q = ok ? rint_to_ll(__fmul_rn(terms[j], kGicpScale)) : 0ll;
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-                        if (lane == j) acc += q;
+                        int hi, lo;
+                        warp_fixed_sum(ok ? terms[j] : 0.0f, hi, lo);
+                        if (lane == j) acc += (long long)hi * 4194304ll + lo;
                     }
                 }
             }
             if (lane < kGicpTerms) atomicAdd(&s_sum[lane], (unsigned long long)acc);
             if (lane == 0) atomicAdd(&s_corr, corr);
             __syncthreads();
-            if (threadIdx.x == 0) {
-                s_last = s_corr;
+            if (warp == 0) {
+                const int n_corr = s_corr;
                 double xi[6];
-                if (s_corr < a.min_corr || !gicp_solve(s_sum, xi)) {
-                    s_done = 1;
-                } else {
-                    if (gicp_update(s_R, s_t, xi, a.stop_rot, a.stop_trans)) s_done = 1;
-                    ++s_updates;
-                    for (int i = 0; i < 9; ++i) s_Rf[i] = __double2float_rn(s_R[i]);
-                    for (int i = 0; i < 3; ++i) s_tf[i] = __double2float_rn(s_t[i]);
+                bool done = true, stepped = false;
+                if (n_corr >= a.min_corr && gicp_solve(s_sum, lane, xi)) {
+                    done = gicp_update(s_R, s_t, xi, a.stop_rot, a.stop_trans, lane);
+                    stepped = true;
+                    if (lane < 9) s_Rf[lane] = __double2float_rn(s_R[lane]);
+                    else if (lane < 12) s_tf[lane - 9] = __double2float_rn(s_t[lane - 9]);
+                }
+                if (lane == 0) {
+                    s_last = n_corr;
+                    s_done = done;
+                    s_updates += stepped;
                 }
             }
             __syncthreads();
