@@ -598,13 +598,26 @@ perch_status perch_load_mesh(perch_ctx* c, const float* verts_xyz, const uint8_t
         dfree(c, rec.verts);
         return st;
     }
+    // the vertices again, sorted for ADD-S, unless the copy would take more than a
+    // small part of what is left of the budget (the unsorted kernel gives the
+    // same errors)
+    std::vector<float> groups;
+    const size_t group_bytes = perch::add_groups_count(n_verts) * sizeof(float4);
+    if (n_verts <= (1 << 28) && (!c->budget || group_bytes <= (c->budget - c->used) / 256)) {
+        groups.resize(group_bytes / sizeof(float));
+        perch::add_groups(v4.data(), n_verts, groups.data());
+        if (dalloc(c, group_bytes, &rec.groups) != PERCH_OK) c->err.clear();
+    }
     cudaError_t e = cudaMemcpyAsync(rec.verts, v4.data(), v4.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && rec.groups)
+        e = cudaMemcpyAsync(rec.groups, groups.data(), groups.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(rec.tris, t4.data(), t4.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         dfree(c, rec.verts);
         dfree(c, rec.tris);
+        dfree(c, rec.groups);
         return cuda_fail(c, e, "perch_load_mesh upload");
     }
     rec.dm.verts = (const float4*)rec.verts;
@@ -637,6 +650,7 @@ perch_status perch_release_mesh(perch_ctx* c, int32_t mesh_id)
     cudaStreamSynchronize(c->stream);
     dfree(c, it->second.verts);
     dfree(c, it->second.tris);
+    dfree(c, it->second.groups);
     c->meshes.erase(it);
     return PERCH_OK;
 }
@@ -1021,9 +1035,15 @@ perch_status perch_add_s(perch_ctx* c, int32_t mesh_id, const float* poses, cons
     if (refuse_while_serving(c) != PERCH_OK) return PERCH_E_BUSY;
     DeviceGuard g(c->device);
     const perch::DevMesh& m = mi->second.dm;
+    const float4* const groups = (const float4*)mi->second.groups;
+    float size = 0.0f;
+    for (int k = 0; k < 3; ++k) size += std::max(std::fabs(m.lo[k]), std::fabs(m.hi[k]));
+    const auto launch = [&](const float* p, const float* t, double* out, cudaStream_t s) {
+        return symmetric && groups ? perch::launch_add_nn(groups, m.n_verts, size, p, t, n, out, s)
+                                   : perch::launch_add_s(m.verts, m.n_verts, p, t, n, symmetric ? 1 : 0, out, s);
+    };
     if (cuda_stream) {
-        cudaError_t e = perch::launch_add_s(m.verts, m.n_verts, poses, poses_true, n, symmetric ? 1 : 0, add,
-                                            (cudaStream_t)cuda_stream);
+        cudaError_t e = launch(poses, poses_true, add, (cudaStream_t)cuda_stream);
         if (e) return cuda_fail(c, e, "perch_add_s");
         return note_async_use(c, -1, mesh_id, (cudaStream_t)cuda_stream);
     }
@@ -1034,7 +1054,7 @@ perch_status perch_add_s(perch_ctx* c, int32_t mesh_id, const float* poses, cons
     double* dout = (double*)((char*)c->stage + (size_t)n * 96);
     cudaError_t e = cudaMemcpyAsync(dp, poses, (size_t)n * 48, cudaMemcpyHostToDevice, c->stream);
     if (!e) e = cudaMemcpyAsync(dt, poses_true, (size_t)n * 48, cudaMemcpyHostToDevice, c->stream);
-    if (!e) e = perch::launch_add_s(m.verts, m.n_verts, dp, dt, n, symmetric ? 1 : 0, dout, c->stream);
+    if (!e) e = launch(dp, dt, dout, c->stream);
     if (!e) e = cudaMemcpyAsync(add, dout, (size_t)n * 8, cudaMemcpyDeviceToHost, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
     return e ? cuda_fail(c, e, "perch_add_s") : PERCH_OK;

@@ -182,6 +182,14 @@ cudaError_t launch_obs_normals(const DevScene& sc, int normal_jump, float4* nrm,
 cudaError_t launch_add_s(const float4* verts, int n_verts, const float* poses, const float* poses_true,
                          long long n, int symmetric, double* out, cudaStream_t s);
 
+// The same ADD-S over vertices sorted into groups of 32 neighbours with bounding
+// spheres: add_groups fills add_groups_count(n) float4 on the host from the
+// packed vertices; size bounds the vertices' norms.
+size_t add_groups_count(int n_verts);
+void add_groups(const float* v4, int n_verts, float* out);
+cudaError_t launch_add_nn(const float4* groups, int n_verts, float size, const float* poses, const float* poses_true,
+                          long long n, double* out, cudaStream_t s);
+
 // Observation build (voxel hash over I).
 struct BuildBuffers {
     // scratch (freed after the build)
