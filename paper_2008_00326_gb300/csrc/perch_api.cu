@@ -296,6 +296,12 @@ perch_status run_jobs(perch_ctx* c, ScoreScratch& X, const std::vector<perch::Jo
     }
     if (total == 0) return PERCH_OK;
     perch::ScoreConfig cfg = cfg_in;
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (!cfg.fixed && total <= kFewPerSm * sms) {
+        cfg.threads = kFewThreads;
+        cfg.zcap_words = kFewZbufWords;
+    }
     perch_status stt = fit_config(c, mark_words, &cfg);
     if (stt != PERCH_OK) return stt;
     const int grid = perch::score_grid(cfg, mark_words);
@@ -966,6 +972,7 @@ perch_status perch_set_launch_config(perch_ctx* c, int32_t threads, int32_t zbuf
     c->cfg.threads = threads;
     c->cfg.zcap_words = zbuf_words & ~3;
     c->cfg.mark_bits = mark_bits;
+    c->cfg.fixed = true;
     return PERCH_OK;
 }
 
@@ -977,6 +984,7 @@ perch_status perch_set_raster_bins(perch_ctx* c, int32_t bin_cap)
     if (bin_cap != 0 && (bin_cap < 64 || bin_cap > 65536))
         return fail(c, PERCH_E_INVALID, "bin capacity %d: 0 or 64 .. 65536", bin_cap);
     c->cfg.bin_cap = bin_cap;
+    c->cfg.fixed = true;
     return PERCH_OK;
 }
 

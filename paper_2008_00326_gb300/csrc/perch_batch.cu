@@ -241,6 +241,7 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
         c->cfg.threads = hit->second.threads;
         c->cfg.zcap_words = hit->second.zcap_words;
         c->cfg.bin_cap = hit->second.bin_cap;
+        c->cfg.fixed = true;
         *threads = c->cfg.threads;
         *zbuf_words = c->cfg.zcap_words;
         if (bin_cap) *bin_cap = c->cfg.bin_cap;
@@ -279,6 +280,7 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
             cfg.threads = th[ti];
             cfg.zcap_words = zw[zi];
             cfg.bin_cap = bc[bi];
+            cfg.fixed = true;
             if (perch::score_smem_bytes(cfg, mw) > 200 * 1024) continue;
             float ms = 3.0e38f;
             for (int rep = 0; rep < 2 && st == PERCH_OK; ++rep) {
@@ -303,6 +305,7 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
     c->cfg.threads = best.threads;
     c->cfg.zcap_words = best.zcap_words;
     c->cfg.bin_cap = best.bin_cap;
+    c->cfg.fixed = true;
     c->tuned[key] = c->cfg;
     *threads = c->cfg.threads;
     *zbuf_words = c->cfg.zcap_words;

@@ -111,6 +111,18 @@ private:
 constexpr int kZbufWordsDefault = 7064;
 constexpr int kMarkBitsDefault = 1 << 15;
 
+// A run of at most two hypotheses per SM, under a launch shape nobody chose,
+// takes blocks of 512 threads (one per SM) and a z-buffer twice as large: its time
+// is that of one or two hypotheses in a row, and 16 warps render and search each
+// faster.  Host to host at 640x480, 512 against 256 threads: 24 poses of a
+// 20,000-triangle mesh 185 against 286 us and of a 30,000-triangle one 329
+// against 580; 304 poses 298 against 317, 556 against 642 and, of a 516-triangle
+// box at 160x120, 177 against 188.  From 400 poses on the smaller blocks win (361
+// against 346, 197 against 187).
+constexpr int kFewPerSm = 2;
+constexpr int kFewThreads = 512;
+constexpr int kFewZbufWords = 14336;
+
 }  // namespace perch_host
 
 struct perch_ctx {

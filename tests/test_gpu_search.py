@@ -28,3 +28,24 @@ def test_candidate_list_sizes(oracle, delta, stride, jo_mode):
     want, _ = oracle.score(oracle.OracleScene.from_scene(sc, **over), oracle.OracleMesh.from_mesh(sc.meshes[0]),
                            poses, label=req.label, roi=req.roi)
     assert np.array_equal(got, want)
+
+
+def test_few_and_many_hypotheses_score_alike():
+    """Runs of up to two hypotheses per SM take larger blocks: the costs are the
+    same on both sides of the line, from one hypothesis up, and under a shape the
+    caller chose."""
+    import torch
+    from paper_2008_00326_gb300 import build, perch as P
+    build.build()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sc = scenes.tabletop_small(colour=True)
+    req = sc.requests[0]
+    with P.Context(0) as ctx:
+        sid, mid = ctx.set_observation(sc), ctx.load_mesh(sc.meshes[0])
+        every = ctx.score(sid, mid, req.label, req.roi, req.poses)
+        assert len(every) > 2 * sms + 1
+        for n in (1, 2, sms, sms + 1, 2 * sms, 2 * sms + 1):
+            assert np.array_equal(ctx.score(sid, mid, req.label, req.roi, req.poses[:n]), every[:n]), n
+        ctx.set_launch_config(128, 2048)
+        for n in (3, 2 * sms + 1):
+            assert np.array_equal(ctx.score(sid, mid, req.label, req.roi, req.poses[:n]), every[:n]), n
