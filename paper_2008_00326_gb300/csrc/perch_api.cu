@@ -38,14 +38,30 @@ perch_status cuda_fail(perch_ctx* c, cudaError_t e, const char* what)
     return fail(c, PERCH_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// Give the observation scratch back (not while it is in use).
+static void drop_build_ws(perch_ctx* c)
+{
+    if (!c->build_ws || c->building) return;
+    void* p = c->build_ws;
+    c->build_ws = nullptr;
+    c->build_ws_bytes = 0;
+    dfree(c, p);
+}
+
 perch_status dalloc(perch_ctx* c, size_t bytes, void** p)
 {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
+    if (c->budget && c->used + bytes > c->budget) drop_build_ws(c);
     if (c->budget && c->used + bytes > c->budget)
         return fail(c, PERCH_E_BUDGET, "allocation of %zu bytes exceeds the HBM budget (%llu of %llu used)",
                     bytes, (unsigned long long)c->used, (unsigned long long)c->budget);
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && c->build_ws && !c->building) {
+        cudaGetLastError();
+        drop_build_ws(c);
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -65,6 +81,17 @@ void dfree(perch_ctx* c, void* p)
         c->allocs.erase(it);
     }
     cudaFree(p);
+}
+
+perch_status ensure_build_ws(perch_ctx* c, size_t bytes)
+{
+    if (c->build_ws_bytes >= bytes) return PERCH_OK;
+    dfree(c, c->build_ws);
+    c->build_ws = nullptr;
+    c->build_ws_bytes = 0;
+    perch_status st = dalloc(c, bytes, &c->build_ws);
+    if (st == PERCH_OK) c->build_ws_bytes = bytes;
+    return st;
 }
 
 perch_status ensure_stage(perch_ctx* c, size_t bytes)
@@ -184,7 +211,7 @@ perch_status make_job(perch_ctx* c, int32_t scene_id, int32_t mesh_id, int32_t l
     auto mi = c->meshes.find(mesh_id);
     if (mi == c->meshes.end()) return fail(c, PERCH_E_NOTFOUND, "unknown mesh %d", mesh_id);
     if (label < -1) return fail(c, PERCH_E_INVALID, "label must be -1 or >= 0");
-    if (label >= 0 && !si->second.labels)
+    if (label >= 0 && !si->second.ds.labels)
         return fail(c, PERCH_E_INVALID, "label %d given but the observation has no labels", label);
     if (n < 0) return fail(c, PERCH_E_INVALID, "n < 0");
     int r[4];
@@ -377,93 +404,145 @@ using namespace perch_host;
 
 namespace {
 
-// Dense cell index over the near-cell box (at most 2^24 cells): the cloud
-// re-sorted by cell (z-major, then y, then x) with each cell's start, so that
-// the radius search reads a row of three cells as one run instead of probing
-// the hash table for each of 27 cells.  The hash table is then no longer
-// needed and is freed.  A larger box keeps the hash table.
-perch_status build_dense_cells(perch_ctx* c, SceneRec& s, long long cells)
+void free_scene(perch_ctx* c, SceneRec& s)
+{
+    dfree(c, s.image); dfree(c, s.index); dfree(c, s.pts); dfree(c, s.table); dfree(c, s.near); dfree(c, s.nrm);
+}
+
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// Dense cell index over the near-cell box (at most 2^24 cells): the cloud sorted
+// by cell (z-major, then y, then x) with each cell's start, so that the radius
+// search reads a row of three cells as one run, and the near-cell bitmap (a bit
+// per cell, set iff one of its 27 neighbours holds a point).
+perch_status build_dense_cells(perch_ctx* c, SceneRec& s, size_t cells)
 {
     perch::DevScene& d = s.ds;
-    d.cell_start = nullptr;
-    if (d.n_pts <= 0 || cells > (1ll << 24)) return PERCH_OK;
-    const size_t n = (size_t)cells, n_tiles = (n + 1023) / 1024;
-    void *count = nullptr, *cursor = nullptr, *sums = nullptr, *out = nullptr;
-    auto cleanup = [&]() { dfree(c, count); dfree(c, cursor); dfree(c, sums); dfree(c, out); };
-    perch_status st;
-    if ((st = dalloc(c, (n + 1) * 4, &s.cstart)) || (st = dalloc(c, n * 4, &count)) ||
-        (st = dalloc(c, n * 4, &cursor)) || (st = dalloc(c, n_tiles * 4, &sums)) ||
-        (st = dalloc(c, (size_t)d.n_pts * sizeof(float4), &out))) {
-        cleanup();
-        dfree(c, s.cstart);
-        s.cstart = nullptr;
-        return st;
-    }
-    const uint32_t last = (uint32_t)d.n_pts;
-    cudaError_t e = cudaMemsetAsync(count, 0, n * 4, c->stream);
-    if (!e) e = cudaMemsetAsync(cursor, 0, n * 4, c->stream);
-    if (!e) e = perch::launch_dense_cells(d, (uint32_t*)count, (uint32_t*)cursor, (uint32_t*)sums,
-                                          (uint32_t*)s.cstart, (float4*)out, c->stream);
-    if (!e) e = cudaMemcpyAsync((uint32_t*)s.cstart + n, &last, 4, cudaMemcpyHostToDevice, c->stream);
+    const size_t tiles = (cells + 1023) / 1024, near_bytes = align256((cells + 31) / 32 * 4);
+    const size_t start_bytes = align256((cells + 1) * 4);
+    perch_status st = dalloc(c, near_bytes + start_bytes + (size_t)d.n_pts * sizeof(float4), &s.index);
+    if (st == PERCH_OK) st = ensure_build_ws(c, (cells + tiles) * 4);
+    if (st != PERCH_OK) return st;
+    c->building = true;
+    uint32_t* const count = (uint32_t*)c->build_ws;
+    uint32_t* const near_bits = (uint32_t*)s.index;
+    uint32_t* const start = (uint32_t*)((char*)s.index + near_bytes);
+    float4* const pts = (float4*)((char*)s.index + near_bytes + start_bytes);
+    cudaError_t e = perch::launch_dense_cells(d, count, count + cells, near_bits, start, pts, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
-    if (e) {
-        cleanup();
-        dfree(c, s.cstart);
-        s.cstart = nullptr;
-        return cuda_fail(c, e, "dense cell index");
-    }
-    dfree(c, count);
-    dfree(c, cursor);
-    dfree(c, sums);
-    dfree(c, s.pts);
-    dfree(c, s.table);
-    s.pts = out;
-    s.table = nullptr;
-    d.pts = (const float4*)out;
-    d.table = nullptr;
-    d.table_mask = 0;
-    d.cell_start = (const uint32_t*)s.cstart;
+    c->building = false;
+    if (e) return cuda_fail(c, e, "dense cell index");
+    d.near_bits = near_bits;
+    d.cell_start = start;
+    d.pts = pts;
     return PERCH_OK;
 }
 
-// Near-cell bitmap of an observation: one bit per hash cell of the observed
-// points' cell box grown by one, set iff one of the cell's 27 neighbours holds
-// a point.  Skipped (no filter) when the box exceeds 2^27 cells.
-perch_status build_near_cells(perch_ctx* c, SceneRec& s)
+// Voxel hash over the cloud, for a cell box too large for the dense index, and
+// the near-cell bitmap when the box has at most 2^27 cells.
+perch_status build_hash(perch_ctx* c, SceneRec& s, const uint8_t* d_rgb, long long cells)
 {
     perch::DevScene& d = s.ds;
-    d.near_bits = nullptr;
-    if (d.n_pts <= 0) return PERCH_OK;
-    void* bnd = nullptr;
-    perch_status st = dalloc(c, 6 * sizeof(int), &bnd);
-    if (st != PERCH_OK) return st;
-    const int init[6] = {INT_MAX, INT_MAX, INT_MAX, INT_MIN, INT_MIN, INT_MIN};
-    int got[6];
-    cudaError_t e = cudaMemcpyAsync(bnd, init, sizeof(init), cudaMemcpyHostToDevice, c->stream);
-    if (!e) e = perch::launch_cell_bounds(d, (int*)bnd, c->stream);
-    if (!e) e = cudaMemcpyAsync(got, bnd, sizeof(got), cudaMemcpyDeviceToHost, c->stream);
+    const long long npx = (long long)d.W * d.H, n_valid = d.n_pts;
+    const uint32_t cap = next_pow2(std::max<long long>(1024, 2 * n_valid)), n_tiles = (cap + 1023) / 1024;
+    perch_status st = PERCH_OK;
+    void *slot = nullptr, *keys = nullptr, *count = nullptr, *cursor = nullptr, *start = nullptr, *nvalid = nullptr,
+         *big = nullptr, *occ = nullptr;
+    auto cleanup = [&](perch_status r) {
+        dfree(c, slot); dfree(c, keys); dfree(c, count); dfree(c, cursor);
+        dfree(c, start); dfree(c, nvalid); dfree(c, big); dfree(c, occ);
+        return r;
+    };
+    if ((st = dalloc(c, std::max<long long>(1, n_valid) * sizeof(float4), &s.pts)) ||
+        (st = dalloc(c, (size_t)cap * sizeof(uint4), &big)) || (st = dalloc(c, npx * sizeof(int32_t), &slot)) ||
+        (st = dalloc(c, (size_t)cap * 8, &keys)) || (st = dalloc(c, (size_t)cap * 4, &count)) ||
+        (st = dalloc(c, ((size_t)cap + n_tiles) * 4, &cursor)) ||
+        (st = dalloc(c, (size_t)cap * 4, &start)) || (st = dalloc(c, 2 * sizeof(int), &nvalid)))
+        return cleanup(st);
+    d.pts = (const float4*)s.pts;
+    d.table = (const uint4*)big;
+    d.table_mask = cap - 1;
+    perch::BuildBuffers b{};
+    b.slot_of_pixel = (int32_t*)slot;
+    b.keys = (unsigned long long*)keys;
+    b.count = (uint32_t*)count;
+    b.cursor = (uint32_t*)cursor;
+    b.start = (uint32_t*)start;
+    b.n_valid = (int*)nvalid;
+    b.lab = const_cast<float4*>(d.lab);
+    b.pxyz = const_cast<float4*>(d.pxyz);
+    b.pts = (float4*)s.pts;
+    b.table = (uint4*)big;
+    cudaError_t e = perch::launch_build(d, b, cap, d_rgb, c->d_err, c->stream);
+    int got[2] = {-1, -1};
+    if (!e) e = cudaMemcpyAsync(got, nvalid, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
-    dfree(c, bnd);
-    if (e) return cuda_fail(c, e, "near-cell bounds");
-    long long cells = 1;
-    for (int a = 0; a < 3; ++a) {
-        d.near_lo[a] = got[a] - 1;
-        d.near_n[a] = got[3 + a] - got[a] + 3;
-        cells *= d.near_n[a];
-    }
-    if (cells > (1ll << 27)) return PERCH_OK;
+    if (e) return cleanup(cuda_fail(c, e, "perch_set_observation build"));
+    if ((st = check_device_error(c)) != PERCH_OK) return cleanup(st);
+    if (got[0] != n_valid)
+        return cleanup(fail(c, PERCH_E_CUDA, "observation build counted %d of %lld points", got[0], n_valid));
+    // compact the hash table to eight times its occupied cells: most of the
+    // 27 lookups per query are misses, and a load factor of at most 1/8 ends
+    // nearly all of them at the first slot
+    const uint32_t cap_small = next_pow2(std::max<long long>(64, 8ll * got[1]));
+    if ((st = dalloc(c, (size_t)cap_small * sizeof(uint4), &s.table)) != PERCH_OK) return cleanup(st);
+    e = perch::launch_compact_table((const uint4*)big, cap, (uint4*)s.table, cap_small, c->d_err, c->stream);
+    if (!e) e = cudaStreamSynchronize(c->stream);
+    if (e) return cleanup(cuda_fail(c, e, "perch_set_observation table"));
+    if ((st = check_device_error(c)) != PERCH_OK) return cleanup(st);
+    d.table = (const uint4*)s.table;
+    d.table_mask = cap_small - 1;
+    if (n_valid == 0 || cells > (1ll << 27)) return cleanup(PERCH_OK);
     const size_t bytes = (size_t)((cells + 31) / 32) * 4;
-    void* occ = nullptr;
-    if ((st = dalloc(c, bytes, &s.near)) != PERCH_OK) return st;
-    if ((st = dalloc(c, bytes, &occ)) != PERCH_OK) return st;
+    if ((st = dalloc(c, bytes, &s.near)) || (st = dalloc(c, bytes, &occ))) return cleanup(st);
     e = cudaMemsetAsync(s.near, 0, bytes, c->stream);
     if (!e) e = cudaMemsetAsync(occ, 0, bytes, c->stream);
     if (!e) e = perch::launch_near_cells(d, (uint32_t*)occ, (uint32_t*)s.near, c->stream);
     if (!e) e = cudaStreamSynchronize(c->stream);
-    dfree(c, occ);
-    if (e) return cuda_fail(c, e, "near-cell bitmap");
+    if (e) return cleanup(cuda_fail(c, e, "near-cell bitmap"));
     d.near_bits = (const uint32_t*)s.near;
-    return build_dense_cells(c, s, cells);
+    return cleanup(PERCH_OK);
+}
+
+// Everything of perch_set_observation that runs on the device: s.ds holds the
+// image, the intrinsics and the parameters.
+perch_status build_observation(perch_ctx* c, SceneRec& s, const uint16_t* depth, const uint8_t* rgb,
+                               const int32_t* labels)
+{
+    perch::DevScene& d = s.ds;
+    const size_t npx = (size_t)d.W * d.H, rgb_bytes = align256(3 * npx), plane = align256(npx * sizeof(float4));
+    const size_t depth_bytes = align256(npx * sizeof(uint16_t));
+    perch_status st = dalloc(c, 2 * plane + depth_bytes + (labels ? npx * sizeof(int32_t) : 0), &s.image);
+    if (st == PERCH_OK) st = ensure_build_ws(c, rgb_bytes + 256);
+    if (st != PERCH_OK) return st;
+    c->building = true;                    // the scratch holds the colours until the index is built
+    char* const at = (char*)s.image;
+    uint8_t* const d_rgb = (uint8_t*)c->build_ws;
+    int* const d_stats = (int*)((char*)c->build_ws + rgb_bytes);
+    d.lab = (const float4*)at;
+    d.pxyz = (const float4*)(at + plane);
+    d.depth = (const uint16_t*)(at + 2 * plane);
+    d.labels = labels ? (const int32_t*)(at + 2 * plane + depth_bytes) : nullptr;
+    int stats[7] = {INT_MAX, INT_MAX, INT_MAX, INT_MIN, INT_MIN, INT_MIN, 0};
+    cudaError_t e = cudaMemcpyAsync(at + 2 * plane, depth, npx * sizeof(uint16_t), cudaMemcpyHostToDevice, c->stream);
+    if (!e) e = cudaMemcpyAsync(d_rgb, rgb, npx * 3, cudaMemcpyHostToDevice, c->stream);
+    if (!e) e = cudaMemcpyAsync(d_stats, stats, sizeof(stats), cudaMemcpyHostToDevice, c->stream);
+    if (!e && labels)
+        e = cudaMemcpyAsync(at + 2 * plane + depth_bytes, labels, npx * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
+    if (!e) e = perch::launch_obs_points(d, d_rgb, (float4*)at, (float4*)(at + plane), d_stats, c->stream);
+    if (!e) e = cudaMemcpyAsync(stats, d_stats, sizeof(stats), cudaMemcpyDeviceToHost, c->stream);
+    if (!e) e = cudaStreamSynchronize(c->stream);
+    if (e) return cuda_fail(c, e, "perch_set_observation build");
+    d.n_pts = stats[6];
+    long long cells = 1;
+    for (int a = 0; a < 3 && d.n_pts > 0; ++a) {
+        d.near_lo[a] = stats[a] - 1;
+        d.near_n[a] = stats[3 + a] - stats[a] + 3;
+        cells *= d.near_n[a];
+    }
+    if (d.n_pts <= 0 || cells > (1ll << 24)) return build_hash(c, s, d_rgb, cells);
+    c->building = false;                   // done with the colours
+    return build_dense_cells(c, s, (size_t)cells);
 }
 
 }  // namespace
@@ -688,46 +767,10 @@ perch_status perch_set_observation(perch_ctx* c, const uint16_t* depth, const ui
         return fail(c, PERCH_E_INVALID, "perch_set_observation: delta too small for the field of view");
 
     std::lock_guard<std::mutex> lk(c->mu);
-    Range r("perch: observation build (cloud, CIELAB, voxel hash)");
-    long long npx = (long long)W * H;
-    long long n_valid = 0;
-    for (long long i = 0; i < npx; ++i) {
-        int u = (int)(i % W), v = (int)(i / W);
-        if (depth[i] != 0 && u % p.stride == 0 && v % p.stride == 0) ++n_valid;
-    }
-    uint32_t cap = next_pow2(std::max<long long>(1024, 2 * n_valid));
-    uint32_t n_tiles = (cap + 1023) / 1024;
-
+    Range r("perch: observation build (cloud, CIELAB, cell index)");
     DeviceGuard g(c->device);
     SceneRec s;
     s.params = p;
-    perch_status st = PERCH_OK;
-    void *d_rgb = nullptr, *slot = nullptr, *keys = nullptr, *count = nullptr, *cursor = nullptr,
-         *start = nullptr, *nvalid = nullptr, *big = nullptr;
-    auto cleanup_scratch = [&]() {
-        dfree(c, d_rgb); dfree(c, slot); dfree(c, keys); dfree(c, count);
-        dfree(c, cursor); dfree(c, start); dfree(c, nvalid); dfree(c, big);
-    };
-    auto cleanup_scene = [&]() {
-        dfree(c, s.depth); dfree(c, s.labels); dfree(c, s.lab); dfree(c, s.pts); dfree(c, s.table); dfree(c, s.nrm);
-        dfree(c, s.near); dfree(c, s.cstart); dfree(c, s.pxyz);
-    };
-    if ((st = dalloc(c, npx * sizeof(uint16_t), &s.depth)) ||
-        (labels && (st = dalloc(c, npx * sizeof(int32_t), &s.labels))) ||
-        (st = dalloc(c, npx * sizeof(float4), &s.lab)) || (st = dalloc(c, npx * sizeof(float4), &s.pxyz)) ||
-        (st = dalloc(c, std::max<long long>(1, n_valid) * sizeof(float4), &s.pts)) ||
-        (st = dalloc(c, (size_t)cap * sizeof(uint4), &big)) ||
-        (st = dalloc(c, npx * 3, &d_rgb)) || (st = dalloc(c, npx * sizeof(int32_t), &slot)) ||
-        (st = dalloc(c, (size_t)cap * 8, &keys)) || (st = dalloc(c, (size_t)cap * 4, &count)) ||
-        (st = dalloc(c, ((size_t)cap + n_tiles) * 4, &cursor)) ||
-        (st = dalloc(c, (size_t)cap * 4, &start)) || (st = dalloc(c, 2 * sizeof(int), &nvalid))) {
-        cleanup_scratch();
-        cleanup_scene();
-        return st;
-    }
-    cudaError_t e = cudaMemcpyAsync(s.depth, depth, npx * sizeof(uint16_t), cudaMemcpyHostToDevice, c->stream);
-    if (!e) e = cudaMemcpyAsync(d_rgb, rgb, npx * 3, cudaMemcpyHostToDevice, c->stream);
-    if (!e && labels) e = cudaMemcpyAsync(s.labels, labels, npx * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
     perch::DevScene& d = s.ds;
     d.W = W; d.H = H; d.fx = fx; d.fy = fy; d.cx = cx; d.cy = cy;
     const bool fast = fx > 0x1p-60f && fx < 0x1p60f && fy > 0x1p-60f && fy < 0x1p60f;
@@ -743,63 +786,11 @@ perch_status perch_set_observation(perch_ctx* c, const uint16_t* depth, const ui
     d.stride = std::min(p.stride, std::max(W, H));   // any larger stride keeps pixel (0, 0) alone too
     d.occ_margin = p.occ_margin_units;
     d.jo_mode = p.jo_mode;
-    d.depth = (const uint16_t*)s.depth;
-    d.labels = (const int32_t*)s.labels;
-    d.lab = (const float4*)s.lab;
-    d.pxyz = (const float4*)s.pxyz;
-    d.pts = (const float4*)s.pts;
-    d.table = (const uint4*)big;
-    d.table_mask = cap - 1;
-    d.n_pts = (int)n_valid;
-    perch::BuildBuffers b{};
-    b.slot_of_pixel = (int32_t*)slot;
-    b.keys = (unsigned long long*)keys;
-    b.count = (uint32_t*)count;
-    b.cursor = (uint32_t*)cursor;
-    b.start = (uint32_t*)start;
-    b.n_valid = (int*)nvalid;
-    b.lab = (float4*)s.lab;
-    b.pxyz = (float4*)s.pxyz;
-    b.pts = (float4*)s.pts;
-    b.table = (uint4*)big;
-    if (!e) e = perch::launch_build(d, b, cap, (const uint8_t*)d_rgb, c->d_err, c->stream);
-    int got[2] = {-1, -1};
-    if (!e) e = cudaMemcpyAsync(got, nvalid, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-    if (!e) e = cudaStreamSynchronize(c->stream);
-    if (e) {
-        cleanup_scratch();
-        cleanup_scene();
-        return cuda_fail(c, e, "perch_set_observation build");
-    }
-    if ((st = check_device_error(c)) != PERCH_OK || got[0] != n_valid) {
-        cleanup_scratch();
-        cleanup_scene();
-        return st != PERCH_OK ? st : fail(c, PERCH_E_CUDA, "observation build counted %d of %lld points", got[0], n_valid);
-    }
-    // compact the hash table to eight times its occupied cells: most of the
-    // 27 lookups per query are misses, and a load factor of at most 1/8 ends
-    // nearly all of them at the first slot
-    uint32_t cap_small = next_pow2(std::max<long long>(64, 8ll * got[1]));
-    if ((st = dalloc(c, (size_t)cap_small * sizeof(uint4), &s.table)) != PERCH_OK) {
-        cleanup_scratch();
-        cleanup_scene();
-        return st;
-    }
-    e = perch::launch_compact_table((const uint4*)big, cap, (uint4*)s.table, cap_small, c->d_err, c->stream);
-    if (!e) e = cudaStreamSynchronize(c->stream);
-    cleanup_scratch();
-    if (e) {
-        cleanup_scene();
-        return cuda_fail(c, e, "perch_set_observation table");
-    }
-    if ((st = check_device_error(c)) != PERCH_OK) {
-        cleanup_scene();
-        return st;
-    }
-    d.table = (const uint4*)s.table;
-    d.table_mask = cap_small - 1;
-    if ((st = build_near_cells(c, s)) != PERCH_OK) {
-        cleanup_scene();
+    const perch_status st = build_observation(c, s, depth, rgb, labels);
+    c->building = false;
+    if (c->build_ws_bytes > kBuildKeep) drop_build_ws(c);
+    if (st != PERCH_OK) {
+        free_scene(c, s);
         return st;
     }
     int32_t id = c->next_id++;
@@ -820,8 +811,7 @@ perch_status perch_release_scene(perch_ctx* c, int32_t scene_id)
         return fail(c, PERCH_E_BUSY, "scene %d is in use (%d served requests or batch graphs, %zu unfinished "
                                      "asynchronous calls)", scene_id, s.use.users, s.use.pending.size());
     cudaStreamSynchronize(c->stream);
-    dfree(c, s.depth); dfree(c, s.labels); dfree(c, s.lab); dfree(c, s.pts); dfree(c, s.table); dfree(c, s.nrm);
-    dfree(c, s.near); dfree(c, s.cstart); dfree(c, s.pxyz);
+    free_scene(c, s);
     c->scenes.erase(it);
     return PERCH_OK;
 }
@@ -1001,7 +991,7 @@ perch_status perch_pose_proposals(perch_ctx* c, int32_t scene_id, int32_t mesh_i
     if (si == c->scenes.end()) return fail(c, PERCH_E_NOTFOUND, "unknown scene %d", scene_id);
     auto mi = c->meshes.find(mesh_id);
     if (mi == c->meshes.end()) return fail(c, PERCH_E_NOTFOUND, "unknown mesh %d", mesh_id);
-    if (label < 0 || !si->second.labels) return fail(c, PERCH_E_INVALID, "proposals need a label and labels");
+    if (label < 0 || !si->second.ds.labels) return fail(c, PERCH_E_INVALID, "proposals need a label and labels");
     if (refuse_while_serving(c) != PERCH_OK) return PERCH_E_BUSY;
     DeviceGuard g(c->device);
     perch::ProposalArgs a{};

@@ -40,16 +40,13 @@ struct MeshRec {
 struct SceneRec {
     perch::DevScene ds{};
     perch_params params{};
-    void* depth = nullptr;
-    void* labels = nullptr;
-    void* lab = nullptr;
-    void* pxyz = nullptr;          // per-pixel observed points (DevScene::pxyz)
-    void* pts = nullptr;
-    void* table = nullptr;
+    void* image = nullptr;         // per pixel: CIELAB, observed point, depth, labels (one allocation)
+    void* index = nullptr;         // dense cell index: near-cell bitmap, cell starts, points by cell
+    void* pts = nullptr;           // voxel hash (a cell box too large for the dense index): points,
+    void* table = nullptr;         // table,
+    void* near = nullptr;          // and near-cell bitmap
     void* nrm = nullptr;           // observed normals (GICP targets), made on first use
     int nrm_jump = -1;             // the normal_max_jump_units they were made with
-    void* near = nullptr;          // near-cell bitmap (DevScene::near_bits)
-    void* cstart = nullptr;        // dense cell index (DevScene::cell_start)
     UseTrack use;
 };
 
@@ -137,6 +134,9 @@ struct perch_ctx {
     cudaStream_t stream = nullptr;
     void* stage = nullptr;
     size_t stage_bytes = 0;
+    void* build_ws = nullptr;                       // scratch of perch_set_observation, kept between calls
+    size_t build_ws_bytes = 0;                      // (up to kBuildKeep) until an allocation needs its room
+    bool building = false;                          // perch_set_observation is using it
     int* d_err = nullptr;
     unsigned long long* d_best_partial = nullptr;   // 3 words per block, kBestMaxBlocks blocks
     unsigned* d_best_ticket = nullptr;
@@ -172,6 +172,10 @@ perch_status cuda_fail(perch_ctx* c, cudaError_t e, const char* what);
 // Device allocation charged to the context's HBM budget; dfree returns it.
 perch_status dalloc(perch_ctx* c, size_t bytes, void** p);
 void dfree(perch_ctx* c, void* p);
+// perch_set_observation's scratch, grown to at least bytes; up to kBuildKeep of
+// it stay allocated when the call ends.
+constexpr size_t kBuildKeep = (size_t)64 << 20;
+perch_status ensure_build_ws(perch_ctx* c, size_t bytes);
 // The context's device staging buffer, grown to at least bytes.
 perch_status ensure_stage(perch_ctx* c, size_t bytes);
 // Read and clear the device error word (synchronous).

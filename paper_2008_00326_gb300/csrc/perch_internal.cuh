@@ -210,15 +210,16 @@ cudaError_t launch_build(const DevScene& sc, const BuildBuffers& b, uint32_t tab
                          const uint8_t* rgb_dev, int* err, cudaStream_t s);
 cudaError_t launch_compact_table(const uint4* big, uint32_t cap_big, uint4* small, uint32_t cap_small,
                                  int* err, cudaStream_t s);
-// Bounding box of the observed points' hash cells: bounds = (min x, y, z, max x, y, z).
-cudaError_t launch_cell_bounds(const DevScene& sc, int* bounds, cudaStream_t s);
+// Per pixel CIELAB and observed point, and stats = (smallest, largest cell
+// coordinates of the points, their count), initialised by the caller.
+cudaError_t launch_obs_points(const DevScene& sc, const uint8_t* rgb, float4* lab, float4* pxyz, int* stats,
+                              cudaStream_t s);
 // Fill sc.near_bits (zeroed) through the occupancy bitmap occ (zeroed, same size).
 cudaError_t launch_near_cells(const DevScene& sc, uint32_t* occ, uint32_t* near_bits, cudaStream_t s);
-// Dense cell index over the near-cell box: cell_start (n_cells + 1 words;
-// the last one is written by the caller) and the points re-sorted by cell
-// into out.  count and cursor (n_cells words each) and tile_sums
-// ((n_cells + 1023) / 1024 words) are zeroed scratch.
-cudaError_t launch_dense_cells(const DevScene& sc, uint32_t* count, uint32_t* cursor, uint32_t* tile_sums,
+// Dense cell index over the near-cell box from sc.pxyz: near_bits, cell_start
+// (n_cells + 1 words) and the points by cell.  count (n_cells words) and tile_sums
+// ((n_cells + 1023) / 1024 words) are scratch.
+cudaError_t launch_dense_cells(const DevScene& sc, uint32_t* count, uint32_t* tile_sums, uint32_t* near_bits,
                                uint32_t* cell_start, float4* out, cudaStream_t s);
 
 // Argmin of J = J_o + J_r (ties to the lowest id / index).  The kernel

@@ -15,6 +15,11 @@
 #include <climits>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <map>
+#include <mutex>
+#include <set>
+#include <tuple>
+#include <utility>
 
 namespace perch {
 
@@ -311,29 +316,6 @@ __global__ void k_compact_table(const uint4* big, uint32_t cap_big, uint4* small
 // ---- near-cell bitmap: lets a query whose 27 neighbour cells are all empty
 // skip the hash lookups (exact: such a query has no candidate at all)
 
-__global__ void k_cell_bounds(DevScene sc, int* bounds)
-{
-    int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sc.n_pts; i += gridDim.x * blockDim.x) {
-        const float4 p = sc.pts[i];
-        const int c[3] = {cell_coord(p.x, sc.inv_cell), cell_coord(p.y, sc.inv_cell), cell_coord(p.z, sc.inv_cell)};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) { lo[a] = min(lo[a], c[a]); hi[a] = max(hi[a], c[a]); }
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo[a] = min(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-            hi[a] = max(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-        }
-    }
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) { atomicMin(&bounds[a], lo[a]); atomicMax(&bounds[3 + a], hi[a]); }
-    }
-}
-
 __device__ __forceinline__ long long near_index(const DevScene& sc, int x, int y, int z)
 {
     const int ix = x - sc.near_lo[0], iy = y - sc.near_lo[1], iz = z - sc.near_lo[2];
@@ -368,13 +350,6 @@ __global__ void k_cell_dilate(DevScene sc, const uint32_t* occ, uint32_t* near_b
     }
 }
 
-cudaError_t launch_cell_bounds(const DevScene& sc, int* bounds, cudaStream_t s)
-{
-    if (sc.n_pts <= 0) return cudaSuccess;
-    k_cell_bounds<<<min(1024, (sc.n_pts + 255) / 256), 256, 0, s>>>(sc, bounds);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_near_cells(const DevScene& sc, uint32_t* occ, uint32_t* near_bits, cudaStream_t s)
 {
     if (sc.n_pts <= 0) return cudaSuccess;
@@ -384,46 +359,146 @@ cudaError_t launch_near_cells(const DevScene& sc, uint32_t* occ, uint32_t* near_
     return cudaGetLastError();
 }
 
-// ---- dense cell index: count per cell, exclusive scan, scatter by cell
+// ---- observation build over the dense cell index: points and their cell box,
+// count per cell, exclusive scan, scatter by cell.  Five small launches read and
+// write each pixel two or three times (the cell arrays, four bytes a cell, are
+// the larger part at a million cells); the hash build they replace for clouds
+// whose cell box is small enough took thirteen.
 
-__global__ void k_dense_count(DevScene sc, uint32_t* count)
+// n / d for 0 <= n < 2^24 and 1 <= d < 2^24 without an integer division: a
+// binary32 estimate (both operands exact, error below one) corrected once.
+__device__ __forceinline__ int div_small(int n, int d)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sc.n_pts; i += gridDim.x * blockDim.x) {
-        const float4 p = sc.pts[i];
-        const long long c = near_index(sc, cell_coord(p.x, sc.inv_cell), cell_coord(p.y, sc.inv_cell),
-                                       cell_coord(p.z, sc.inv_cell));
-        if (c >= 0) atomicAdd(&count[c], 1u);
-    }
+    int q = __float2int_rz(__fmul_rn(__int2float_rn(n), __frcp_rn(__int2float_rn(d))));
+    const int r = n - q * d;
+    q += (r >= d) - (r < 0);
+    return q;
 }
 
-__global__ void k_add_tile_offsets(uint32_t* start, const uint32_t* tile_offsets, uint32_t n)
+__device__ __forceinline__ bool on_lattice(const DevScene& sc, int u, int v)
+{
+    return div_small(u, sc.stride) * sc.stride == u && div_small(v, sc.stride) * sc.stride == v;
+}
+
+// Per pixel CIELAB and observed point; stats = (smallest, largest cell
+// coordinates of the points, their count), initialised to (INT_MAX x 3,
+// INT_MIN x 3, 0).
+__global__ void __launch_bounds__(256) k_obs_points(DevScene sc, const uint8_t* __restrict__ rgb, float4* lab,
+                                                   float4* pxyz, int* stats)
+{
+    __shared__ int red[7];
+    if (threadIdx.x < 7) red[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : threadIdx.x < 6 ? INT_MIN : 0;
+    __syncthreads();
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    int c[3] = {INT_MAX, INT_MAX, INT_MAX};
+    bool in = false;
+    if (i < sc.W * sc.H) {
+        const int v = div_small(i, sc.W), u = i - v * sc.W;
+        const float3 L = srgb8_to_lab(rgb[3 * i], rgb[3 * i + 1], rgb[3 * i + 2]);
+        lab[i] = make_float4(L.x, L.y, L.z, 0.0f);
+        const unsigned d = sc.depth[i];
+        in = d != 0 && on_lattice(sc, u, v);
+        float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (in) {
+            const float3 q = back_project(sc, u, v, d);
+            p = make_float4(q.x, q.y, q.z, 1.0f);
+            c[0] = cell_coord(q.x, sc.inv_cell);
+            c[1] = cell_coord(q.y, sc.inv_cell);
+            c[2] = cell_coord(q.z, sc.inv_cell);
+        }
+        pxyz[i] = p;
+    }
+    const unsigned any = __ballot_sync(0xffffffffu, in);
+    if (any != 0u) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int lo = __reduce_min_sync(0xffffffffu, c[a]), hi = __reduce_max_sync(0xffffffffu, in ? c[a] : INT_MIN);
+            if ((threadIdx.x & 31) == 0) {
+                atomicMin(&red[a], lo);
+                atomicMax(&red[3 + a], hi);
+            }
+        }
+        if ((threadIdx.x & 31) == 0) atomicAdd(&red[6], __popc(any));
+    }
+    __syncthreads();
+    if (red[6] == 0) return;
+    if (threadIdx.x < 3) atomicMin(&stats[threadIdx.x], red[threadIdx.x]);
+    else if (threadIdx.x < 6) atomicMax(&stats[threadIdx.x], red[threadIdx.x]);
+    else if (threadIdx.x == 6) atomicAdd(&stats[6], red[6]);
+}
+
+// Linear cell of an observed point (its cell lies inside the box's border).
+__device__ __forceinline__ int point_cell(const DevScene& sc, float4 p)
+{
+    const int x = cell_coord(p.x, sc.inv_cell) - sc.near_lo[0], y = cell_coord(p.y, sc.inv_cell) - sc.near_lo[1];
+    const int z = cell_coord(p.z, sc.inv_cell) - sc.near_lo[2];
+    return (z * sc.near_n[1] + y) * sc.near_n[0] + x;
+}
+
+// Points per cell; the first point of a cell marks the cell's 27 neighbours, nine
+// rows of three consecutive bits, in the near-cell bitmap (both arrays zeroed).
+__global__ void __launch_bounds__(256) k_cell_count(DevScene sc, uint32_t* count, uint32_t* near_bits)
+{
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= sc.W * sc.H) return;
+    const float4 p = sc.pxyz[i];
+    if (p.w == 0.0f) return;
+    const int c = point_cell(sc, p);
+    if (atomicAdd(&count[c], 1u) != 0u) return;
+    const int nx = sc.near_n[0], nxy = nx * sc.near_n[1];
+    for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy) {
+            const int b = c + dz * nxy + dy * nx - 1;
+            atomicOr(&near_bits[b >> 5], 7u << (b & 31));
+            if ((b & 31) > 29) atomicOr(&near_bits[(b >> 5) + 1], 7u >> (32 - (b & 31)));
+        }
+}
+
+// start[i] += its tile's offset; start[n] = total.
+__global__ void k_add_tile_offsets(uint32_t* start, const uint32_t* tile_offsets, uint32_t n, uint32_t total)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) start[i] += tile_offsets[i >> 10];
+    else if (i == n) start[n] = total;
 }
 
-__global__ void k_dense_scatter(DevScene sc, const uint32_t* start, uint32_t* cursor, float4* out)
+// The points by cell (any order within a cell: a nearest neighbour's ties go by
+// pixel); count runs down to zero.
+__global__ void __launch_bounds__(256) k_cell_scatter(DevScene sc, const uint32_t* start, uint32_t* count, float4* out)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < sc.n_pts; i += gridDim.x * blockDim.x) {
-        const float4 p = sc.pts[i];
-        const long long c = near_index(sc, cell_coord(p.x, sc.inv_cell), cell_coord(p.y, sc.inv_cell),
-                                       cell_coord(p.z, sc.inv_cell));
-        if (c >= 0) out[start[c] + atomicAdd(&cursor[c], 1u)] = p;
-    }
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= sc.W * sc.H) return;
+    float4 p = sc.pxyz[i];
+    if (p.w == 0.0f) return;
+    const int c = point_cell(sc, p), v = div_small(i, sc.W);
+    // the pixel as (v << 16 | u): ordered like the index v W + u, and its
+    // coordinates come back without a division
+    p.w = __uint_as_float(((uint32_t)v << 16) | (uint32_t)(i - v * sc.W));
+    out[start[c] + atomicSub(&count[c], 1u) - 1u] = p;
 }
 
-cudaError_t launch_dense_cells(const DevScene& sc, uint32_t* count, uint32_t* cursor, uint32_t* tile_sums,
+cudaError_t launch_obs_points(const DevScene& sc, const uint8_t* rgb, float4* lab, float4* pxyz, int* stats,
+                              cudaStream_t s)
+{
+    k_obs_points<<<(sc.W * sc.H + 255) / 256, 256, 0, s>>>(sc, rgb, lab, pxyz, stats);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dense_cells(const DevScene& sc, uint32_t* count, uint32_t* tile_sums, uint32_t* near_bits,
                                uint32_t* cell_start, float4* out, cudaStream_t s)
 {
     const long long n = (long long)sc.near_n[0] * sc.near_n[1] * sc.near_n[2];
-    if (sc.n_pts <= 0 || n <= 0 || n > 0xFFFFFFFFll) return cudaErrorInvalidValue;
-    const unsigned blocks_pts = (unsigned)std::min(1024, (sc.n_pts + 255) / 256);
-    k_dense_count<<<blocks_pts, 256, 0, s>>>(sc, count);
+    if (sc.n_pts <= 0 || n <= 0 || n > 0x7FFFFFFFll) return cudaErrorInvalidValue;
+    const unsigned blocks = (unsigned)((sc.W * sc.H + 255) / 256);
+    cudaError_t e = cudaMemsetAsync(count, 0, (size_t)n * 4, s);
+    if (!e) e = cudaMemsetAsync(near_bits, 0, (size_t)((n + 31) / 32) * 4, s);
+    if (e) return e;
+    k_cell_count<<<blocks, 256, 0, s>>>(sc, count, near_bits);
     const uint32_t n_tiles = (uint32_t)((n + 1023) / 1024);
     k_scan_tiles<<<n_tiles, 1024, 0, s>>>(count, cell_start, tile_sums, (uint32_t)n);
     k_scan_sums<<<1, 1024, 0, s>>>(tile_sums, n_tiles);
-    k_add_tile_offsets<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(cell_start, tile_sums, (uint32_t)n);
-    k_dense_scatter<<<blocks_pts, 256, 0, s>>>(sc, cell_start, cursor, out);
+    k_add_tile_offsets<<<(unsigned)(n / 256 + 1), 256, 0, s>>>(cell_start, tile_sums, (uint32_t)n, (uint32_t)sc.n_pts);
+    k_cell_scatter<<<blocks, 256, 0, s>>>(sc, cell_start, count, out);
     return cudaGetLastError();
 }
 
@@ -1169,16 +1244,6 @@ __device__ __forceinline__ bool get_triangle(const DevScene& sc, const DevMesh& 
                                              const unsigned long long* vc, int t, TriSetup& o)
 {
     return load_tri<VC>(sc, m, P, vc, __ldg(&m.tris[t]), o) && orient_triangle(o);
-}
-
-// n / d for 0 <= n < 2^24 and 1 <= d < 2^24 without an integer division: a
-// binary32 estimate (both operands exact, error below one) corrected once.
-__device__ __forceinline__ int div_small(int n, int d)
-{
-    int q = __float2int_rz(__fmul_rn(__int2float_rn(n), __frcp_rn(__int2float_rn(d))));
-    const int r = n - q * d;
-    q += (r >= d) - (r < 0);
-    return q;
 }
 
 // ---- rasteriser: rings of triangles and covered samples --------------------
@@ -2179,15 +2244,34 @@ size_t score_smem_bytes(const ScoreConfig& cfg, int mark_words)
     return smem_layout(cfg.zcap_words, mark_words, cfg.threads).total;
 }
 
+// Let fn use all the shared memory a block may have, once per device: the limit
+// is a property of the function, so calls that set it to what each needs would
+// undercut one another between threads (and cost a driver call per launch).
+static cudaError_t allow_smem(const void* fn)
+{
+    static std::mutex mu;
+    static std::set<std::pair<int, const void*>> done;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(mu);
+    if (done.count({dev, fn})) return cudaSuccess;
+    cudaFuncAttributes fa{};
+    e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) done.insert({dev, fn});
+    return e;
+}
+
 template <int NT, int MODE, bool BINS>
 static int score_grid_nt(size_t smem)
 {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaFuncSetAttribute(k_score<NT, MODE, BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return -1;
+    if (allow_smem((const void*)k_score<NT, MODE, BINS>) != cudaSuccess) return -1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_score<NT, MODE, BINS>, NT, smem) != cudaSuccess)
         return -1;
     return max(1, per) * max(1, sms);
@@ -2208,12 +2292,20 @@ static int score_grid_all(size_t smem)
 
 int score_grid(const ScoreConfig& cfg, int mark_words)
 {
-    size_t smem = score_smem_bytes(cfg, mark_words);
-    switch (cfg.threads) {
-    case 128: return score_grid_all<128>(smem);
-    case 512: return score_grid_all<512>(smem);
-    default: return score_grid_all<256>(smem);
-    }
+    // a function of the device and the shape alone, asked for on every call
+    static std::mutex mu;
+    static std::map<std::tuple<int, int, size_t>, int> known;
+    const size_t smem = score_smem_bytes(cfg, mark_words);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const std::tuple<int, int, size_t> key(dev, cfg.threads, smem);
+    std::lock_guard<std::mutex> lk(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    const int g = cfg.threads == 128 ? score_grid_all<128>(smem)
+                                     : cfg.threads == 512 ? score_grid_all<512>(smem) : score_grid_all<256>(smem);
+    if (g > 0 && known.size() < 4096) known[key] = g;
+    return g;
 }
 
 // a with the places of the block's shared-memory regions, which the kernel reads
@@ -2244,7 +2336,7 @@ static cudaError_t launch_score_nt(const ScoreArgs& a, const ScoreConfig& cfg, i
     const size_t smem = score_smem_bytes(cfg, a.mark_words);
     const unsigned g = (unsigned)(a.n < grid ? a.n : grid);
     const void* fn = score_kernel<NT>(a);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess) return e;
     ScoreArgs copy = with_layout(a, NT);
     void* args[] = {&copy};
@@ -2258,7 +2350,7 @@ static cudaError_t add_score_node_nt(cudaGraph_t g, const cudaGraphNode_t* deps,
 {
     const size_t smem = score_smem_bytes(cfg, a.mark_words);
     const void* fn = score_kernel<NT>(a);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(fn);
     if (e != cudaSuccess) return e;
     ScoreArgs copy = with_layout(a, NT);
     void* args[] = {&copy};
@@ -2797,9 +2889,7 @@ int gicp_grid(int zcap_words)
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = gicp_smem_bytes(zcap_words);
-    if (cudaFuncSetAttribute(k_gicp<kGicpThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return -1;
+    if (allow_smem((const void*)k_gicp<kGicpThreads>) != cudaSuccess) return -1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_gicp<kGicpThreads>, kGicpThreads, smem) != cudaSuccess)
         return -1;
     return max(1, per) * max(1, sms);
@@ -2810,7 +2900,7 @@ cudaError_t launch_gicp(const GicpArgs& a, int grid, cudaStream_t s)
     if (a.n <= 0) return cudaSuccess;
     if (a.n > 0xFFFFFFF0ll || grid <= 0 || grid > a.slots) return cudaErrorInvalidValue;
     const size_t smem = gicp_smem_bytes(a.zcap_words);
-    cudaError_t e = cudaFuncSetAttribute(k_gicp<kGicpThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void*)k_gicp<kGicpThreads>);
     if (e != cudaSuccess) return e;
     k_gicp<kGicpThreads><<<(unsigned)(a.n < grid ? a.n : grid), kGicpThreads, smem, s>>>(a);
     return cudaGetLastError();
