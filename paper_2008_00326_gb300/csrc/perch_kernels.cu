@@ -1,5 +1,5 @@
 // libperch kernels for sm_103a: observation build (back-projection, CIELAB,
-// voxel hash over I), the fused per-hypothesis scorer (fixed-point raster with
+// cell index over I), the fused per-hypothesis scorer (fixed-point raster with
 // an atomicMin z-buffer in shared memory, resolve with occluder removal and
 // image-space down-sampling, warp-cooperative 27-cell radius search,
 // CIEDE2000 check, J_r / J_o counts) and the warp-shuffle argmin.
@@ -1142,6 +1142,14 @@ struct ScoreSmem {
     int* vbounds;                 // snapped vertex bounds of the hypothesis (vertex_pass)
 };
 
+// rint(x) for |x| < 2^22: adding 1.5 x 2^23 rounds to an integer, ties to even,
+// and leaves it in the low bits (a conversion holds its unit for eight issue
+// slots; the vertex pass is a sixteenth of a search).
+__device__ __forceinline__ int rint_small(float x)
+{
+    return __float_as_int(__fadd_rn(x, 12582912.0f)) - 0x4B400000;
+}
+
 // ---- per-hypothesis vertex cache (one slot of global scratch per block) ----
 //
 // Each vertex is transformed, projected and snapped once per hypothesis and
@@ -1153,7 +1161,6 @@ struct ScoreSmem {
 constexpr int kSnapBias = 1 << 14;            // 1024 pixels in 1/16 px
 constexpr uint32_t kCulledXY = 0xFFFFFFFFu;
 
-//
 // bounds (optional, shared memory, initialised to INT_MAX, INT_MAX, INT_MIN,
 // INT_MIN): the smallest and largest snapped x and y of the vertices kept.
 __device__ __forceinline__ void vertex_pass(const DevScene& sc, const DevMesh& m, const float* P,
@@ -1175,7 +1182,8 @@ __device__ __forceinline__ void vertex_pass(const DevScene& sc, const DevMesh& m
         if (Z >= sc.z_near) {
             const float iz = __frcp_rn(Z);
             float xz, yz;
-            if (div_fits(X) && div_fits(Y) && Z > kDivLo && Z < kDivHi) {
+            const float small = fminf(fabsf(X), fminf(fabsf(Y), Z)), large = fmaxf(fabsf(X), fmaxf(fabsf(Y), Z));
+            if (small > kDivLo && large < kDivHi) {
                 xz = div_by(X, Z, iz);
                 yz = div_by(Y, Z, iz);
             } else {
@@ -1185,7 +1193,7 @@ __device__ __forceinline__ void vertex_pass(const DevScene& sc, const DevMesh& m
             const float sx = __fmul_rn(__fadd_rn(__fmul_rn(sc.fx, xz), sc.cx), 16.0f);
             const float sy = __fmul_rn(__fadd_rn(__fmul_rn(sc.fy, yz), sc.cy), 16.0f);
             if (sx >= gx0 && sx < gx1 && sy >= gy0 && sy < gy1) {
-                const int xi = __float2int_rn(sx), yi = __float2int_rn(sy);
+                const int xi = rint_small(sx), yi = rint_small(sy);
                 xmin = min(xmin, xi); xmax = max(xmax, xi);
                 ymin = min(ymin, yi); ymax = max(ymax, yi);
                 rec = (unsigned long long)((uint32_t)(xi + kSnapBias) | ((uint32_t)(yi + kSnapBias) << 16)) |
