@@ -527,7 +527,7 @@ perch_status build_observation(perch_ctx* c, SceneRec& s, const uint16_t* depth,
     if (st != PERCH_OK) return st;
     c->building = true;                    // the scratch holds the colours until the index is built
     char* const at = (char*)s.image;
-    uint8_t* const d_rgb = (uint8_t*)c->build_ws;
+    uint8_t* d_rgb = (uint8_t*)c->build_ws;
     int* const d_stats = (int*)((char*)c->build_ws + rgb_bytes);
     d.lab = (const float4*)at;
     d.pxyz = (const float4*)(at + plane);
@@ -550,7 +550,20 @@ perch_status build_observation(perch_ctx* c, SceneRec& s, const uint16_t* depth,
         d.near_n[a] = stats[3 + a] - stats[a] + 3;
         cells *= d.near_n[a];
     }
-    if (d.n_pts <= 0 || cells > (1ll << 24)) return build_hash(c, s, d_rgb, cells);
+    if (d.n_pts <= 0 || cells > (1ll << 24)) {
+        if (c->budget && c->build_ws_bytes > rgb_bytes + 256) {
+            // a larger scratch, kept by an earlier build, would take the hash's room in
+            // the budget: hold the colours alone
+            c->building = false;
+            drop_build_ws(c);
+            if ((st = ensure_build_ws(c, rgb_bytes + 256)) != PERCH_OK) return st;
+            c->building = true;
+            d_rgb = (uint8_t*)c->build_ws;
+            e = cudaMemcpyAsync(d_rgb, rgb, npx * 3, cudaMemcpyHostToDevice, c->stream);
+            if (e) return cuda_fail(c, e, "perch_set_observation build");
+        }
+        return build_hash(c, s, d_rgb, cells);
+    }
     c->building = false;                   // done with the colours
     return build_dense_cells(c, s, (size_t)cells);
 }

@@ -89,3 +89,33 @@ def test_scratch_is_given_back(P):
             P.perch_release_scene(ctx.ctx, s)
         assert ctx.hbm_used <= used
         ctx.set_observation(sc)
+
+
+def test_kept_scratch_leaves_the_hash_its_room(P):
+    rng = np.random.default_rng(2)
+    depth = rng.integers(5200, 6600, (60, 80)).astype(np.uint16)
+    depth[::7, ::5] = 30000
+    rgb = np.zeros((60, 80, 3), np.uint8)
+
+    def build(ctx, delta):
+        return P.perch_set_observation(ctx.ctx, depth, rgb, None, 150.0, 150.0, 40.0, 30.0,
+                                       P.perch_default_params(delta_m=delta, color_check=0))
+
+    def fits(budget):
+        try:
+            with P.Context(0, hbm_budget_bytes=budget) as ctx:
+                build(ctx, 0.005)               # some 38 million cells: the hash
+            return True
+        except P.PerchError as e:
+            assert e.status == -3
+            return False
+
+    lo, hi = 1 << 20, 64 << 20
+    assert fits(hi)
+    while hi - lo > 32 << 10:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid) else (mid, hi)
+    with P.Context(0, hbm_budget_bytes=hi) as ctx:
+        sid = build(ctx, 0.018)                 # some 0.8 million cells: 3.3 MB of scratch stay
+        P.perch_release_scene(ctx.ctx, sid)
+        build(ctx, 0.005)
