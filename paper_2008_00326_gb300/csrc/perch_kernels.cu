@@ -3008,98 +3008,151 @@ cudaError_t launch_proposals(const ProposalArgs& a, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------------------
-// argmin of J = J_o + J_r (warp shuffles, then the last block reduces the partials)
+// argmin of J = J_o + J_r (the last block reduces the blocks' results)
 // ---------------------------------------------------------------------------
-
+//
+// Bound by latency, not by bytes: a launch is one or a few rounds of loads, the
+// block's reduction, the ticket and the last block's reduction in a row.  So the
+// costs are read first, kBestUnroll pairs in flight per thread, and only a thread
+// that holds the block's smallest J reads an id (all of its equal ones, in a second
+// pass over its pairs, when it holds several); reductions are warp-wide integer
+// minima of 32 bits, one per part of the key.  A call in a queue of calls, with
+// ids: 500 pairs 4.1 us (6.2 with one pair in flight per thread, every id read and
+// 64-bit shuffles), 300,001 pairs 6.2 (9.2), 2,000,000 pairs 8.2 (12.3) and, all
+// equal, 10.3 (13.3).
 constexpr int kBestThreads = 256;
+constexpr int kBestUnroll = 4;
+constexpr int kBestGrid = 4 * 152;       // blocks at most: four per SM
+static_assert(kBestGrid <= kBestMaxBlocks, "a block's result has its place in the scratch");
 
 struct BestKey {
-    unsigned long long hi;   // (J << 32) | 0
+    unsigned J;              // compared as unsigned, like the upper half of the packed key
     unsigned long long id;   // caller id or index
-    long long idx;
+    unsigned idx;            // below 2^31; the key of nothing has all bits set
 };
 
-__device__ __forceinline__ bool best_less(const BestKey& x, const BestKey& y)
+__device__ __forceinline__ BestKey best_none() { return {0xFFFFFFFFu, ~0ull, 0xFFFFFFFFu}; }
+
+// The smallest key of the warp's lanes by (J, id, index), in every lane.
+__device__ __forceinline__ BestKey warp_best(const BestKey& k)
 {
-    if (x.hi != y.hi) return x.hi < y.hi;
-    if (x.id != y.id) return x.id < y.id;
-    return x.idx < y.idx;
+    const unsigned full = 0xffffffffu, hi = (unsigned)(k.id >> 32), lo = (unsigned)k.id;
+    const unsigned J = __reduce_min_sync(full, k.J);
+    const unsigned h = __reduce_min_sync(full, k.J == J ? hi : full);
+    const unsigned l = __reduce_min_sync(full, k.J == J && hi == h ? lo : full);
+    const unsigned x = __reduce_min_sync(full, k.J == J && hi == h && lo == l ? k.idx : full);
+    return {J, ((unsigned long long)h << 32) | l, x};
 }
 
-__device__ __forceinline__ BestKey shfl_best(const BestKey& k, int o)
+// The smallest key of the block's threads (in every lane of every warp).
+__device__ __forceinline__ BestKey block_best(BestKey k, BestKey* sh)
 {
-    BestKey r;
-    r.hi = __shfl_xor_sync(0xffffffffu, k.hi, o);
-    r.id = __shfl_xor_sync(0xffffffffu, k.id, o);
-    r.idx = __shfl_xor_sync(0xffffffffu, k.idx, o);
-    return r;
-}
-
-__device__ BestKey block_best(BestKey k, BestKey* sh)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        BestKey t = shfl_best(k, o);
-        if (best_less(t, k)) k = t;
-    }
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sh[w] = k;
+    const int lane = threadIdx.x & 31;
+    k = warp_best(k);
+    if (lane == 0) sh[threadIdx.x >> 5] = k;
     __syncthreads();
-    if (w == 0) {
-        BestKey none = {~0ull, ~0ull, 0x7FFFFFFFFFFFFFFFll};
-        k = lane < kBestThreads / 32 ? sh[lane] : none;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            BestKey t = shfl_best(k, o);
-            if (best_less(t, k)) k = t;
-        }
+    return warp_best(lane < kBestThreads / 32 ? sh[lane] : best_none());
+}
+
+// J of pair i (its low 32 bits); costs may be aligned to 4 bytes only.
+__device__ __forceinline__ unsigned pair_cost(const BestArgs& a, bool wide, long long i)
+{
+    if (wide) {
+        const int2 c = reinterpret_cast<const int2*>(a.costs)[i];
+        return (unsigned)c.x + (unsigned)c.y;
     }
-    return k;
+    return (unsigned)a.costs[2 * i] + (unsigned)a.costs[2 * i + 1];
 }
 
 __global__ void __launch_bounds__(kBestThreads) k_best(BestArgs a)
 {
-    __shared__ BestKey sh[kBestThreads / 32];
+    __shared__ BestKey sh[2][kBestThreads / 32];
+    __shared__ unsigned low[kBestThreads / 32];
     __shared__ bool last;
-    BestKey k = {~0ull, ~0ull, 0x7FFFFFFFFFFFFFFFll};
-    for (long long i = blockIdx.x * (long long)kBestThreads + threadIdx.x; i < a.n;
-         i += (long long)gridDim.x * kBestThreads) {
-        long long J = (long long)a.costs[2 * i] + a.costs[2 * i + 1];
-        BestKey c = {(unsigned long long)J << 32, a.ids ? a.ids[i] : (unsigned long long)i, i};
-        if (best_less(c, k)) k = c;
+    const bool wide = (reinterpret_cast<uintptr_t>(a.costs) & 7) == 0;
+    const long long first = blockIdx.x * (long long)(kBestThreads * kBestUnroll) + threadIdx.x;
+    const long long step = gridDim.x * (long long)(kBestThreads * kBestUnroll);
+    unsigned best = 0xFFFFFFFFu, at = 0xFFFFFFFFu;    // smallest J and the first index that has it
+    bool ties = false;
+    for (long long b = first; b < a.n; b += step) {
+        unsigned J[kBestUnroll];
+#pragma unroll
+        for (int u = 0; u < kBestUnroll; ++u)
+            J[u] = b + u * kBestThreads < a.n ? pair_cost(a, wide, b + u * kBestThreads) : 0xFFFFFFFFu;
+#pragma unroll
+        for (int u = 0; u < kBestUnroll; ++u) {
+            const long long i = b + u * kBestThreads;
+            if (i >= a.n) continue;
+            if (J[u] < best || at == 0xFFFFFFFFu) {
+                best = J[u];
+                at = (unsigned)i;
+                ties = false;
+            } else if (J[u] == best) {
+                ties = true;
+            }
+        }
     }
-    k = block_best(k, sh);
-    if (threadIdx.x == 0) {
-        a.partial[3 * blockIdx.x + 0] = k.hi;
-        a.partial[3 * blockIdx.x + 1] = k.id;
-        a.partial[3 * blockIdx.x + 2] = (unsigned long long)k.idx;
+    const unsigned w = __reduce_min_sync(0xffffffffu, best);
+    if ((threadIdx.x & 31) == 0) low[threadIdx.x >> 5] = w;
+    __syncthreads();
+    unsigned m = low[0];
+#pragma unroll
+    for (int i = 1; i < kBestThreads / 32; ++i) m = min(m, low[i]);
+    BestKey k = best_none();
+    if (best == m && at != 0xFFFFFFFFu) {
+        k = {m, a.ids ? a.ids[at] : (unsigned long long)at, at};
+        if (a.ids && ties) {
+            for (long long b = first; b < a.n; b += step) {
+                unsigned long long id[kBestUnroll];
+                bool eq[kBestUnroll];
+#pragma unroll
+                for (int u = 0; u < kBestUnroll; ++u) {
+                    const long long i = b + u * kBestThreads;
+                    eq[u] = i < a.n && pair_cost(a, wide, i) == m;
+                    id[u] = eq[u] ? a.ids[i] : ~0ull;
+                }
+#pragma unroll
+                for (int u = 0; u < kBestUnroll; ++u)      // indices ascend: the first of equal ids stays
+                    if (eq[u] && id[u] < k.id) {
+                        k.id = id[u];
+                        k.idx = (unsigned)(b + u * kBestThreads);
+                    }
+            }
+        }
+    }
+    k = block_best(k, sh[0]);
+    if (gridDim.x > 1) {
+        if (threadIdx.x == 0) {
+            a.partial[3 * blockIdx.x + 0] = k.J;
+            a.partial[3 * blockIdx.x + 1] = k.id;
+            a.partial[3 * blockIdx.x + 2] = k.idx;
+            __threadfence();
+            last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+        }
+        __syncthreads();
+        if (!last) return;
         __threadfence();
-        unsigned t = atomicAdd(a.ticket, 1u);
-        last = (t == gridDim.x - 1);
+        k = best_none();
+        for (unsigned b = threadIdx.x; b < gridDim.x; b += kBestThreads) {
+            const volatile unsigned long long* const p = a.partial + 3 * b;
+            const BestKey c = {(unsigned)p[0], p[1], (unsigned)p[2]};
+            if (c.J < k.J || (c.J == k.J && (c.id < k.id || (c.id == k.id && c.idx < k.idx)))) k = c;
+        }
+        k = block_best(k, sh[1]);
+        if (threadIdx.x == 0) *a.ticket = 0u;
     }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    BestKey m = {~0ull, ~0ull, 0x7FFFFFFFFFFFFFFFll};
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kBestThreads) {
-        BestKey c = {a.partial[3 * b], a.partial[3 * b + 1], (long long)a.partial[3 * b + 2]};
-        if (best_less(c, m)) m = c;
-    }
-    __syncthreads();
-    m = block_best(m, sh);
     if (threadIdx.x == 0) {
-        if (a.best_index) *a.best_index = m.idx;
-        if (a.best_cost) *a.best_cost = (int32_t)(m.hi >> 32);
+        if (a.best_index) *a.best_index = k.idx;
+        if (a.best_cost) *a.best_cost = (int32_t)k.J;
         // (J << 32) | id: the smallest such key over several shards is their winner
-        if (a.key) *a.key = m.hi | (m.id & 0xFFFFFFFFull);
-        *a.ticket = 0u;
+        if (a.key) *a.key = ((unsigned long long)k.J << 32) | (k.id & 0xFFFFFFFFull);
     }
 }
 
 int best_blocks(long long n)
 {
-    long long b = (n + kBestThreads - 1) / kBestThreads;
-    return (int)(b < 1 ? 1 : (b > kBestMaxBlocks ? kBestMaxBlocks : b));
+    const long long b = (n + kBestThreads * kBestUnroll - 1) / (kBestThreads * kBestUnroll);
+    return (int)(b < 1 ? 1 : (b > kBestGrid ? kBestGrid : b));
 }
 
 cudaError_t launch_best(const BestArgs& a, cudaStream_t s)
