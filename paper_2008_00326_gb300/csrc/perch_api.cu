@@ -131,17 +131,17 @@ uint32_t next_pow2(uint64_t x)
 
 perch_status clip_roi(perch_ctx* c, const SceneRec& s, const int32_t* roi, int out[4])
 {
-    int W = s.ds.W, H = s.ds.H;
+    const int W = s.ds.W, H = s.ds.H;
     if (!roi) {
         out[0] = 0; out[1] = 0; out[2] = W; out[3] = H;
         return PERCH_OK;
     }
-    out[0] = std::max(0, roi[0]);
-    out[1] = std::max(0, roi[1]);
-    out[2] = std::min(W, roi[2]);
-    out[3] = std::min(H, roi[3]);
-    if (out[2] < out[0]) out[2] = out[0];
-    if (out[3] < out[1]) out[3] = out[1];
+    // every bound inside the image, an empty box included: the kernels pack pixels
+    // into 16 bits and divide by binary32 estimates that hold up to 2^24
+    out[0] = std::min(std::max(0, roi[0]), W);
+    out[1] = std::min(std::max(0, roi[1]), H);
+    out[2] = std::max(out[0], std::min(W, roi[2]));
+    out[3] = std::max(out[1], std::min(H, roi[3]));
     (void)c;
     return PERCH_OK;
 }

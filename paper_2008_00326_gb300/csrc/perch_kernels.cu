@@ -1780,8 +1780,9 @@ __device__ __forceinline__ void score_tiles(const ScoreArgs& a, const Job& J, co
             __syncthreads();
             // (the depth rings take the place of the kept-point queues, idle meanwhile)
             const bool in_bin = BINS && binned && S.bin_cnt[tile] <= a.bin_cap;
-            raster<NT, K32, VC>(sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw, a.err,
-                                in_bin ? bins + tile * a.bin_cap : nullptr, in_bin ? S.bin_cnt[tile] : 0);
+            if (MODE != kModePlain || (rw > 0 && rh > 0))
+                raster<NT, K32, VC>(sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw, a.err,
+                                    in_bin ? bins + tile * a.bin_cap : nullptr, in_bin ? S.bin_cnt[tile] : 0);
             __syncthreads();
             if (a.dump) {
                 for (int i = threadIdx.x; i < tpx; i += NT) {
