@@ -174,18 +174,14 @@ perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg)
     return PERCH_OK;
 }
 
-void default_shape(const perch_ctx* c, const std::vector<perch::Job>& jobs, long long total, perch::ScoreConfig* cfg)
+void default_shape(const perch_ctx* c, long long total, perch::ScoreConfig* cfg)
 {
     if (cfg->fixed) return;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    long long image = 0;
-    for (const auto& j : jobs) image = std::max(image, (long long)j.sc.W * j.sc.H);
     if (total <= kFewPerSm * sms) {
         cfg->threads = kFewThreads;
         cfg->zcap_words = kFewZbufWords;
-    } else if (image <= kSmallImage) {
-        cfg->zcap_words = kSmallZbufWords;
     }
 }
 
@@ -338,7 +334,7 @@ perch_status run_jobs(perch_ctx* c, ScoreScratch& X, const std::vector<perch::Jo
     }
     if (total == 0) return PERCH_OK;
     perch::ScoreConfig cfg = cfg_in;
-    default_shape(c, jobs, total, &cfg);
+    default_shape(c, total, &cfg);
     perch_status stt = fit_config(c, mark_words, &cfg);
     if (stt != PERCH_OK) return stt;
     const int grid = perch::score_grid(cfg, mark_words);

@@ -120,14 +120,6 @@ constexpr int kFewPerSm = 2;
 constexpr int kFewThreads = 512;
 constexpr int kFewZbufWords = 14336;
 
-// Renders in images of up to 320x240 fit a smaller z-buffer, and with 4,864 words
-// four blocks leave 60 KB of an SM to the L1 cache instead of 28 (968 poses at
-// 160x120: 90.0 against 94.4 us; sixteen 320x240 scenes: 112.9 against 115.1 ms).
-// At 640x480 a fifth of the 6-DoF renders would take a second tile (19.1 against
-// 18.9 ms).
-constexpr long long kSmallImage = 320 * 240;
-constexpr int kSmallZbufWords = 4864;
-
 }  // namespace perch_host
 
 struct perch_ctx {
@@ -195,7 +187,7 @@ int mark_words_for(const SceneRec& s, int label, const int roi[4], int cap_bits)
 perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg);
 // The launch shape of a run of `total` hypotheses when neither the caller nor the
 // autotuner has chosen one.
-void default_shape(const perch_ctx* c, const std::vector<perch::Job>& jobs, long long total, perch::ScoreConfig* cfg);
+void default_shape(const perch_ctx* c, long long total, perch::ScoreConfig* cfg);
 perch_status scratch_init(perch_ctx* c, ScoreScratch& X);
 void scratch_free(perch_ctx* c, ScoreScratch& X);
 // PERCH_E_BUSY (with a message) while a server runs on the context.

@@ -2,12 +2,12 @@
 wholly past it: the box is empty, with its bounds inside the image, which is what the
 kernels' 16-bit pixels and binary32 divisions are made for.  Host code only: the
 library's own clip_roi, called from a small C++ program."""
-import os
-import shutil
 import subprocess
 
 import numpy as np
 import pytest
+
+from host_program import build_program
 
 PROGRAM = r"""
 #include "perch_host.cuh"
@@ -28,17 +28,7 @@ int main()
 
 @pytest.fixture(scope="module")
 def clip(tmp_path_factory):
-    from paper_2008_00326_gb300 import build
-    build.build()
-    objs = [os.path.join(build.BUILD_DIR, s.replace(".cu", ".o")) for s in build.SOURCES]
-    if not all(os.path.exists(o) for o in objs):
-        build.build(force=True)
-    d = tmp_path_factory.mktemp("clip")
-    src, exe = d / "clip.cpp", str(d / "clip")
-    src.write_text(PROGRAM)
-    cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or build._nvcc()))
-    subprocess.check_call([build._nvcc(), "-std=c++17", "-I", build.INCLUDE, "-I", build.CSRC,
-                           "-I", os.path.join(cuda, "include"), str(src), *objs, "-o", exe])
+    exe = build_program(tmp_path_factory.mktemp("clip"), PROGRAM)
 
     def run(W, H, rois):
         text = "\n".join(" ".join(str(int(x)) for x in (W, H, *r)) for r in rois)
