@@ -179,7 +179,7 @@ void default_shape(const perch_ctx* c, long long total, perch::ScoreConfig* cfg)
     if (cfg->fixed) return;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (total <= kFewPerSm * sms) {
+    if (total * kFewShare <= sms) {
         cfg->threads = kFewThreads;
         cfg->zcap_words = kFewZbufWords;
     }

@@ -108,15 +108,18 @@ private:
 constexpr int kZbufWordsDefault = 7064;
 constexpr int kMarkBitsDefault = 1 << 15;
 
-// A run of at most two hypotheses per SM, under a launch shape nobody chose,
-// takes blocks of 512 threads (one per SM) and a z-buffer twice as large: its time
-// is that of one or two hypotheses in a row, and 16 warps render and search each
-// faster.  Host to host at 640x480, 512 against 256 threads: 24 poses of a
-// 20,000-triangle mesh 185 against 286 us and of a 30,000-triangle one 329
-// against 580; 304 poses 298 against 317, 556 against 642 and, of a 516-triangle
-// box at 160x120, 177 against 188.  From 400 poses on the smaller blocks win (361
-// against 346, 197 against 187).
-constexpr int kFewPerSm = 2;
+// A run of at most one hypothesis for every second SM, under a launch shape nobody
+// chose, takes blocks of 512 threads (one per SM: 128 registers a thread) and a
+// z-buffer twice as large: its time is that of one hypothesis, and 16 warps render
+// and search it faster.  The line: two such runs of different contexts or server
+// slots still have an SM for each block; past it the 256-thread blocks, four to an
+// SM, overlap more.  us a search with several contexts in flight, 512 / 256 threads:
+// 76 poses 309 / 644 (30,000 triangles, 640x480), 45 / 65 (3,000, 360x260, stride 2)
+// and 34.8 / 38.9 (2,900, 181x127, stride 2); 117 poses 366 / 703, 62 / 70 and 51.0 /
+// 40.7; 300 poses 891 / 866, 147 / 87 and 113 / 48.  8 to 76 poses in each of one to
+// eight contexts: 0.94 (Eq. 3, eight contexts) to 2.0 times the rate.  Host to host, 24
+// poses of a 20,000-triangle mesh at 640x480: 184 / 287.
+constexpr int kFewShare = 2;
 constexpr int kFewThreads = 512;
 constexpr int kFewZbufWords = 14336;
 
