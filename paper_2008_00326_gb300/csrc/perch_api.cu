@@ -159,30 +159,37 @@ int mark_words_for(const SceneRec& s, int label, const int roi[4], int cap_bits)
     return (int)(((bits + 31) / 32 + 2) & ~1ll);   // even: keeps the later 8-byte arrays aligned
 }
 
+// Shared memory that a block of the context's device may have.
+static size_t block_smem(const perch_ctx* c)
+{
+    int max_optin = 0;
+    cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    return max_optin > 0 ? (size_t)max_optin : 48 * 1024;
+}
+
 // Shrink the z-buffer of *cfg (the caller's launch shape) until the block's
 // shared memory fits the device's opt-in limit.
 perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg)
 {
-    int max_optin = 0;
-    cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    if (max_optin <= 0) max_optin = 48 * 1024;
-    while (perch::score_smem_bytes(*cfg, mark_words) > (size_t)max_optin && cfg->zcap_words > 1024)
+    const size_t limit = block_smem(c);
+    while (perch::score_smem_bytes(*cfg, mark_words) > limit && cfg->zcap_words > 1024)
         cfg->zcap_words /= 2;
-    if (perch::score_smem_bytes(*cfg, mark_words) > (size_t)max_optin)
+    if (perch::score_smem_bytes(*cfg, mark_words) > limit)
         return fail(c, PERCH_E_INVALID, "admissible-set bitset (%d words) does not fit in shared memory",
                     mark_words);
     return PERCH_OK;
 }
 
-void default_shape(const perch_ctx* c, long long total, perch::ScoreConfig* cfg)
+void default_shape(const perch_ctx* c, long long total, int mark_words, perch::ScoreConfig* cfg)
 {
     if (cfg->fixed) return;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (total * kFewShare <= sms) {
-        cfg->threads = kFewThreads;
-        cfg->zcap_words = kFewZbufWords;
-    }
+    perch::ScoreConfig few = *cfg;
+    few.threads = kFewThreads;
+    few.zcap_words = kFewZbufWords;
+    // (its 16 warps' scratch leaves less for wide images' marks than the base shape's)
+    if (total * kFewShare <= sms && perch::score_smem_bytes(few, mark_words) <= block_smem(c)) *cfg = few;
 }
 
 perch_status scratch_init(perch_ctx* c, ScoreScratch& X)
@@ -334,7 +341,7 @@ perch_status run_jobs(perch_ctx* c, ScoreScratch& X, const std::vector<perch::Jo
     }
     if (total == 0) return PERCH_OK;
     perch::ScoreConfig cfg = cfg_in;
-    default_shape(c, total, &cfg);
+    default_shape(c, total, mark_words, &cfg);
     perch_status stt = fit_config(c, mark_words, &cfg);
     if (stt != PERCH_OK) return stt;
     const int grid = perch::score_grid(cfg, mark_words);

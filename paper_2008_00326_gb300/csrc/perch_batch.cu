@@ -103,7 +103,7 @@ perch_status perch_batch_graph_create(perch_ctx* c, const perch_work_item* items
     if (st != PERCH_OK) return st;
     if (total == 0) return fail(c, PERCH_E_INVALID, "empty batch");
     perch::ScoreConfig cfg = c->cfg;
-    default_shape(c, total, &cfg);
+    default_shape(c, total, mw, &cfg);
     if ((st = fit_config(c, mw, &cfg)) != PERCH_OK) return st;
     const int resident = perch::score_grid(cfg, mw);
     if (resident <= 0) {

@@ -190,7 +190,7 @@ int mark_words_for(const SceneRec& s, int label, const int roi[4], int cap_bits)
 perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg);
 // The launch shape of a run of `total` hypotheses when neither the caller nor the
 // autotuner has chosen one.
-void default_shape(const perch_ctx* c, long long total, perch::ScoreConfig* cfg);
+void default_shape(const perch_ctx* c, long long total, int mark_words, perch::ScoreConfig* cfg);
 perch_status scratch_init(perch_ctx* c, ScoreScratch& X);
 void scratch_free(perch_ctx* c, ScoreScratch& X);
 // PERCH_E_BUSY (with a message) while a server runs on the context.

@@ -49,3 +49,25 @@ def test_short_runs_end_at_half_the_sms(P, jo_mode):
         assert few[1] != base[1]
         assert used == (few if 2 * n <= sms else base)[1], n
         assert np.array_equal(costs, few[0]) and np.array_equal(costs, base[0]), n
+
+
+def test_short_runs_on_wide_images(P, oracle):
+    """Eq. 3's keys of one image row leave room for the scratch of eight warps, not of
+    sixteen: a run of a few poses takes the shape of a longer one."""
+    H, W, f = 4, 23000, 100.0
+    rng = np.random.default_rng(3)
+    depth = rng.integers(5850, 6050, (H, W)).astype(np.uint16)
+    rgb = np.zeros((H, W, 3), np.uint8)
+    mesh = scenes.box_mesh(0.3, 0.015, 0.015, 30, 3, 3)
+    pose = np.array([1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0.59], np.float32)
+    step = np.float32(0.05) * (np.arange(12) == 3) - np.float32(0.02) * (np.arange(12) == 11)
+    poses = np.stack([pose + k * step for k in range(3)]).astype(np.float32)
+    over = dict(color_check=0, stride=1, jo_mode=1)
+    with P.Context(0) as ctx:
+        mid = ctx.load_mesh(mesh)
+        sid = P.perch_set_observation(ctx.ctx, depth, rgb, None, f, f, W / 2.0, H / 2.0,
+                                      P.perch_default_params(delta_m=0.01, **over))
+        got = ctx.score(sid, mid, -1, None, poses)
+    osc = oracle.OracleScene(depth, rgb, None, f, f, W / 2.0, H / 2.0, delta=0.01, **over)
+    want, _ = oracle.score(osc, oracle.OracleMesh.from_mesh(mesh), poses)
+    assert want[:, 1].max() > want[:, 1].min() and np.array_equal(got, want)

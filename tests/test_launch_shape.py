@@ -18,7 +18,7 @@ int main()
 {
     perch_ctx c;
     perch::ScoreConfig cfg = c.cfg;
-    default_shape(&c, 100000, &cfg);
+    default_shape(&c, 100000, 1026, &cfg);
     print("long", cfg);
 }
 """
