@@ -247,9 +247,10 @@ PERCH_API perch_status perch_best_noalloc(const int32_t *costs, const uint64_t *
  * default 32768).  Pixel boxes larger than the z-buffer are processed in
  * tiles, admissible boxes larger than the bitset in row bands.  Results do not
  * depend on these choices; only speed and shared memory do.  A new context
- * uses 256 threads, 7064 words and 32768 bits (four blocks per SM).  The
- * autotuner of the batched form calls it.  PERCH_E_INVALID outside the
- * ranges. */
+ * uses 256 threads, 7064 words and 32768 bits (four blocks per SM), and for
+ * runs of up to half as many hypotheses as the device has SMs 512 threads and
+ * 14336 words; a shape set here holds for runs of every size.  The autotuner
+ * of the batched form sets one too.  PERCH_E_INVALID outside the ranges. */
 PERCH_API perch_status perch_set_launch_config(perch_ctx *ctx, int32_t threads, int32_t zbuf_words,
                                                int32_t mark_bits);
 
@@ -316,8 +317,9 @@ PERCH_API perch_status perch_batch_graph_destroy(perch_batch_graph *g);
  * context's launch configuration and remember it for batches of the same
  * class (largest ROI area and triangle count, each rounded to a power of
  * two); a later call for a known class returns the remembered shape without
- * timing.  *threads, *zbuf_words and *bin_cap (may be NULL) receive the
- * choice. */
+ * timing.  A shape timed on more hypotheses than half the device's SMs holds
+ * for runs of more than that.  *threads, *zbuf_words and *bin_cap (may be
+ * NULL) receive the choice. */
 PERCH_API perch_status perch_autotune(perch_ctx *ctx, const perch_work_item *items, int32_t n_items,
                                       const float *poses, int32_t *costs, int32_t *threads,
                                       int32_t *zbuf_words, int32_t *bin_cap);

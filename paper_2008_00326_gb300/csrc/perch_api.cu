@@ -180,16 +180,29 @@ perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg)
     return PERCH_OK;
 }
 
+bool short_run(const perch_ctx* c, long long total)
+{
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    return total * kFewShare <= sms;
+}
+
 void default_shape(const perch_ctx* c, long long total, int mark_words, perch::ScoreConfig* cfg)
 {
     if (cfg->fixed) return;
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     perch::ScoreConfig few = *cfg;
     few.threads = kFewThreads;
     few.zcap_words = kFewZbufWords;
     // (its 16 warps' scratch leaves less for wide images' marks than the base shape's)
-    if (total * kFewShare <= sms && perch::score_smem_bytes(few, mark_words) <= block_smem(c)) *cfg = few;
+    if (short_run(c, total) && perch::score_smem_bytes(few, mark_words) <= block_smem(c)) *cfg = few;
+}
+
+void adopt_tuned(perch_ctx* c, const perch::ScoreConfig& best, bool short_too)
+{
+    c->cfg.threads = best.threads;
+    c->cfg.zcap_words = best.zcap_words;
+    c->cfg.bin_cap = best.bin_cap;
+    c->cfg.fixed = short_too;
 }
 
 perch_status scratch_init(perch_ctx* c, ScoreScratch& X)
@@ -1000,7 +1013,6 @@ perch_status perch_set_raster_bins(perch_ctx* c, int32_t bin_cap)
     if (bin_cap != 0 && (bin_cap < 64 || bin_cap > 65536))
         return fail(c, PERCH_E_INVALID, "bin capacity %d: 0 or 64 .. 65536", bin_cap);
     c->cfg.bin_cap = bin_cap;
-    c->cfg.fixed = true;
     return PERCH_OK;
 }
 

@@ -225,7 +225,7 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
     if (rs != PERCH_OK) return rs;
     DeviceGuard g(c->device);
     // class of the batch: largest ROI area and triangle count, as powers of two
-    long long max_area = 0, max_tris = 0;
+    long long max_area = 0, max_tris = 0, hyps = 0;
     for (int32_t i = 0; i < n_items; ++i) {
         auto si = c->scenes.find(items[i].scene_id);
         auto mi = c->meshes.find(items[i].mesh_id);
@@ -235,14 +235,12 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
                              : (long long)si->second.ds.W * si->second.ds.H;
         max_area = std::max(max_area, area);
         max_tris = std::max<long long>(max_tris, mi->second.dm.n_tris);
+        hyps += std::max<long long>(0, items[i].n);
     }
     const uint64_t key = ((uint64_t)next_pow2(max_area) << 32) | next_pow2(max_tris);
     auto hit = c->tuned.find(key);
     if (hit != c->tuned.end()) {
-        c->cfg.threads = hit->second.threads;
-        c->cfg.zcap_words = hit->second.zcap_words;
-        c->cfg.bin_cap = hit->second.bin_cap;
-        c->cfg.fixed = true;
+        adopt_tuned(c, hit->second, hit->second.fixed);
         *threads = c->cfg.threads;
         *zbuf_words = c->cfg.zcap_words;
         if (bin_cap) *bin_cap = c->cfg.bin_cap;
@@ -303,10 +301,7 @@ perch_status perch_autotune(perch_ctx* c, const perch_work_item* items, int32_t 
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != PERCH_OK) return st;
-    c->cfg.threads = best.threads;
-    c->cfg.zcap_words = best.zcap_words;
-    c->cfg.bin_cap = best.bin_cap;
-    c->cfg.fixed = true;
+    adopt_tuned(c, best, short_run(c, hyps));
     c->tuned[key] = c->cfg;
     *threads = c->cfg.threads;
     *zbuf_words = c->cfg.zcap_words;

@@ -188,9 +188,14 @@ uint32_t next_pow2(uint64_t x);
 perch_status clip_roi(perch_ctx* c, const SceneRec& s, const int32_t* roi, int out[4]);
 int mark_words_for(const SceneRec& s, int label, const int roi[4], int cap_bits);
 perch_status fit_config(perch_ctx* c, int mark_words, perch::ScoreConfig* cfg);
+// Is a run of `total` hypotheses one of the short ones (kFewShare)?
+bool short_run(const perch_ctx* c, long long total);
 // The launch shape of a run of `total` hypotheses when neither the caller nor the
 // autotuner has chosen one.
 void default_shape(const perch_ctx* c, long long total, int mark_words, perch::ScoreConfig* cfg);
+// Make `best`, the fastest shape on a batch, the context's: for every run if the
+// batch was a short run (short_too), else for the longer runs only.
+void adopt_tuned(perch_ctx* c, const perch::ScoreConfig& best, bool short_too);
 perch_status scratch_init(perch_ctx* c, ScoreScratch& X);
 void scratch_free(perch_ctx* c, ScoreScratch& X);
 // PERCH_E_BUSY (with a message) while a server runs on the context.

@@ -129,7 +129,7 @@ struct ScoreConfig {
     int zcap_words;           // z-buffer words (32-bit keys: pixels; 64-bit: half)
     int mark_bits;            // admissible-box bitset capacity in bits
     int bin_cap;              // triangles per z-buffer tile bin, 0 = no bins
-    bool fixed = false;       // set by the caller or the autotuner: used as it is for every size of run
+    bool fixed = false;       // chosen by the caller or the autotuner for short runs too
 };
 
 // 8-byte words of one vertex-cache slot: the vertex records, then (bin_cap > 0)
