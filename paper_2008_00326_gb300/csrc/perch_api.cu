@@ -324,7 +324,8 @@ void count_users(perch_ctx* c, int32_t scene_id, int32_t mesh_id, int d)
 static void free_tracking(UseTrack& u)
 {
     for (cudaEvent_t ev : u.pending) {
-        cudaEventSynchronize(ev);
+        // (an event recorded under capture cannot be waited for: no error to leave behind)
+        if (cudaEventSynchronize(ev) != cudaSuccess) cudaGetLastError();
         cudaEventDestroy(ev);
     }
     u.pending.clear();
