@@ -15,6 +15,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <new>
 
 namespace perch_host {
 
@@ -531,6 +532,51 @@ perch_status build_hash(perch_ctx* c, SceneRec& s, const uint8_t* d_rgb, long lo
     return cleanup(PERCH_OK);
 }
 
+// The mesh's vertices sorted for ADD-S, for a call on stream s: made on the mesh's
+// first symmetric call (copied back, sorted on the host and uploaded: 1.1 ms at 10,001
+// vertices), so that neither loading a mesh nor a server that shares the context's
+// lock pays for it.  nullptr: the call takes the kernel over all pairs, whose means
+// differ by the order of their binary64 sum alone.  A captured call does too: what
+// it may allocate and wait for is nothing.
+const float4* add_s_groups(perch_ctx* c, MeshRec& rec, cudaStream_t s)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    const int nv = rec.dm.n_verts;
+    if (rec.groups || nv > (1 << 28)) return (const float4*)rec.groups;
+    const size_t bytes = perch::add_groups_count(nv) * sizeof(float4);
+    if (c->budget && bytes > (c->budget - c->used) / 256) return nullptr;
+    Range r("perch: ADD-S vertex groups");
+    void* p = nullptr;
+    if (dalloc(c, bytes, &p) != PERCH_OK) {
+        c->err.clear();
+        return nullptr;
+    }
+    cudaError_t e = cudaSuccess;
+    try {
+        std::vector<float> v4((size_t)nv * 4), groups(bytes / sizeof(float));
+        e = cudaMemcpyAsync(v4.data(), rec.verts, v4.size() * sizeof(float), cudaMemcpyDeviceToHost, c->stream);
+        if (!e) e = cudaStreamSynchronize(c->stream);
+        if (!e) {
+            perch::add_groups(v4.data(), nv, groups.data());
+            e = cudaMemcpyAsync(p, groups.data(), bytes, cudaMemcpyHostToDevice, c->stream);
+        }
+        if (!e) e = cudaStreamSynchronize(c->stream);
+    } catch (const std::bad_alloc&) {
+        e = cudaErrorMemoryAllocation;
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        dfree(c, p);
+        return nullptr;
+    }
+    rec.groups = p;
+    return (const float4*)p;
+}
+
 // Everything of perch_set_observation that runs on the device: s.ds holds the
 // image, the intrinsics and the parameters.
 perch_status build_observation(perch_ctx* c, SceneRec& s, const uint16_t* depth, const uint8_t* rgb,
@@ -723,26 +769,13 @@ perch_status perch_load_mesh(perch_ctx* c, const float* verts_xyz, const uint8_t
         dfree(c, rec.verts);
         return st;
     }
-    // the vertices again, sorted for ADD-S, unless the copy would take more than a
-    // small part of what is left of the budget (the unsorted kernel gives the
-    // same errors)
-    std::vector<float> groups;
-    const size_t group_bytes = perch::add_groups_count(n_verts) * sizeof(float4);
-    if (n_verts <= (1 << 28) && (!c->budget || group_bytes <= (c->budget - c->used) / 256)) {
-        groups.resize(group_bytes / sizeof(float));
-        perch::add_groups(v4.data(), n_verts, groups.data());
-        if (dalloc(c, group_bytes, &rec.groups) != PERCH_OK) c->err.clear();
-    }
     cudaError_t e = cudaMemcpyAsync(rec.verts, v4.data(), v4.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess && rec.groups)
-        e = cudaMemcpyAsync(rec.groups, groups.data(), groups.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(rec.tris, t4.data(), t4.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         dfree(c, rec.verts);
         dfree(c, rec.tris);
-        dfree(c, rec.groups);
         return cuda_fail(c, e, "perch_load_mesh upload");
     }
     rec.dm.verts = (const float4*)rec.verts;
@@ -1072,12 +1105,13 @@ perch_status perch_add_s(perch_ctx* c, int32_t mesh_id, const float* poses, cons
     if (refuse_while_serving(c) != PERCH_OK) return PERCH_E_BUSY;
     DeviceGuard g(c->device);
     const perch::DevMesh& m = mi->second.dm;
-    const float4* const groups = (const float4*)mi->second.groups;
+    const float4* const groups = symmetric ? add_s_groups(c, mi->second, cuda_stream ? (cudaStream_t)cuda_stream : c->stream)
+                                           : nullptr;
     float size = 0.0f;
     for (int k = 0; k < 3; ++k) size += std::max(std::fabs(m.lo[k]), std::fabs(m.hi[k]));
     const auto launch = [&](const float* p, const float* t, double* out, cudaStream_t s) {
-        return symmetric && groups ? perch::launch_add_nn(groups, m.n_verts, size, p, t, n, out, s)
-                                   : perch::launch_add_s(m.verts, m.n_verts, p, t, n, symmetric ? 1 : 0, out, s);
+        return groups ? perch::launch_add_nn(groups, m.n_verts, size, p, t, n, out, s)
+                      : perch::launch_add_s(m.verts, m.n_verts, p, t, n, symmetric ? 1 : 0, out, s);
     };
     if (cuda_stream) {
         cudaError_t e = launch(poses, poses_true, add, (cudaStream_t)cuda_stream);

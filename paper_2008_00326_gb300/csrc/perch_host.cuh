@@ -33,7 +33,7 @@ struct MeshRec {
     perch::DevMesh dm{};
     void* verts = nullptr;
     void* tris = nullptr;
-    void* groups = nullptr;        // vertices sorted for ADD-S (perch::add_groups), or nullptr: did not fit
+    void* groups = nullptr;        // vertices sorted for ADD-S (perch::add_groups), made by the first call that uses them
     UseTrack use;
 };
 

@@ -1,0 +1,68 @@
+"""The sorted copy of a mesh's vertices that ADD-S reads: made by the first call that
+uses it and charged to the budget then; a captured call does without it."""
+import numpy as np
+import pytest
+
+from paper_2008_00326_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    from paper_2008_00326_gb300 import build, perch
+    build.build()
+    perch.load()
+    return perch
+
+
+def pairs(n, seed=4):
+    rng = np.random.default_rng(seed)
+    true = np.empty((n, 3, 4))
+    true[:, :, :3] = scenes.rodrigues_batch(rng.normal(size=(n, 3)), rng.uniform(0, 3, n))
+    true[:, :, 3] = rng.normal(size=(n, 3)) * 0.1 + [0, 0, 0.9]
+    est = true.copy()
+    est[:, :, :3] = scenes.rodrigues_batch(rng.normal(size=(n, 3)), rng.normal(size=n) * 0.2) @ est[:, :, :3]
+    est[:, :, 3] += rng.normal(size=(n, 3)) * 0.01
+    return est.reshape(n, 12).astype(np.float32), true.reshape(n, 12).astype(np.float32)
+
+
+MESH = scenes.ellipsoid_mesh(0.04, 0.03, 0.05, 41, 40)
+
+
+def test_made_by_the_first_call_that_uses_it(P):
+    est, true = pairs(5)
+    nv, nt = len(MESH.verts), len(MESH.tris)
+    with P.Context(0) as ctx:
+        before = ctx.hbm_used
+        mid = ctx.load_mesh(MESH)
+        assert ctx.hbm_used == before + 16 * (nv + nt)      # vertices and triangles, nothing else
+        P.perch_add_s(ctx.ctx, mid, est, true, False)
+        used = ctx.hbm_used
+        P.perch_add_s(ctx.ctx, mid, est, true, True)
+        assert ctx.hbm_used == used + 16 * 33 * -(-nv // 32)
+        P.perch_add_s(ctx.ctx, mid, est, true, True)
+        assert ctx.hbm_used == used + 16 * 33 * -(-nv // 32)
+        P.perch_release_mesh(ctx.ctx, mid)
+        assert ctx.hbm_used == used - 16 * (nv + nt)
+
+
+def test_captured_calls(P):
+    import torch
+    est, true = pairs(7)
+    dev = [torch.from_numpy(x).cuda() for x in (est, true)]
+    out = torch.zeros(7, dtype=torch.float64, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with P.Context(0) as ctx:
+        mid = ctx.load_mesh(MESH)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            P.perch_add_s(ctx.ctx, mid, *dev, True, out=out, stream=stream)
+        for _ in range(2):                                  # before and after the copy exists
+            graph.replay()
+            torch.cuda.synchronize()
+            got = out.cpu().numpy()
+            np.testing.assert_allclose(got, P.perch_add_s(ctx.ctx, mid, est, true, True), rtol=1e-13)
+            out.zero_()
+        del graph
