@@ -49,18 +49,34 @@ static void drop_build_ws(perch_ctx* c)
     dfree(c, p);
 }
 
+// Give the meshes' sorted copies for ADD-S back, once the calls that read them have
+// ended (later ones make them again, or do without).
+static void drop_add_s_groups(perch_ctx* c)
+{
+    for (auto& kv : c->meshes) {
+        MeshRec& m = kv.second;
+        if (!m.groups) continue;
+        for (cudaEvent_t ev : m.use.pending)
+            if (cudaEventSynchronize(ev) != cudaSuccess) cudaGetLastError();
+        dfree(c, m.groups);
+        m.groups = nullptr;
+    }
+}
+
 perch_status dalloc(perch_ctx* c, size_t bytes, void** p)
 {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     if (c->budget && c->used + bytes > c->budget) drop_build_ws(c);
+    if (c->budget && c->used + bytes > c->budget) drop_add_s_groups(c);
     if (c->budget && c->used + bytes > c->budget)
         return fail(c, PERCH_E_BUDGET, "allocation of %zu bytes exceeds the HBM budget (%llu of %llu used)",
                     bytes, (unsigned long long)c->used, (unsigned long long)c->budget);
     cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaSuccess && c->build_ws && !c->building) {
+    if (e != cudaSuccess) {
         cudaGetLastError();
         drop_build_ws(c);
+        drop_add_s_groups(c);
         e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) {
@@ -536,8 +552,8 @@ perch_status build_hash(perch_ctx* c, SceneRec& s, const uint8_t* d_rgb, long lo
 // first symmetric call (copied back, sorted on the host and uploaded: 1.1 ms at 10,001
 // vertices), so that neither loading a mesh nor a server that shares the context's
 // lock pays for it.  nullptr: the call takes the kernel over all pairs, whose means
-// differ by the order of their binary64 sum alone.  A captured call does too: what
-// it may allocate and wait for is nothing.
+// differ by the order of their binary64 sum alone.  A captured call does too: it may
+// not allocate or wait, and may be replayed after the copy has been given back.
 const float4* add_s_groups(perch_ctx* c, MeshRec& rec, cudaStream_t s)
 {
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -548,7 +564,8 @@ const float4* add_s_groups(perch_ctx* c, MeshRec& rec, cudaStream_t s)
     const int nv = rec.dm.n_verts;
     if (rec.groups || nv > (1 << 28)) return (const float4*)rec.groups;
     const size_t bytes = perch::add_groups_count(nv) * sizeof(float4);
-    if (c->budget && bytes > (c->budget - c->used) / 256) return nullptr;
+    // (no other mesh's copy makes room for this one)
+    if (c->budget && c->used - c->build_ws_bytes + bytes > c->budget) return nullptr;
     Range r("perch: ADD-S vertex groups");
     void* p = nullptr;
     if (dalloc(c, bytes, &p) != PERCH_OK) {
@@ -1105,11 +1122,11 @@ perch_status perch_add_s(perch_ctx* c, int32_t mesh_id, const float* poses, cons
     if (refuse_while_serving(c) != PERCH_OK) return PERCH_E_BUSY;
     DeviceGuard g(c->device);
     const perch::DevMesh& m = mi->second.dm;
-    const float4* const groups = symmetric ? add_s_groups(c, mi->second, cuda_stream ? (cudaStream_t)cuda_stream : c->stream)
-                                           : nullptr;
     float size = 0.0f;
     for (int k = 0; k < 3; ++k) size += std::max(std::fabs(m.lo[k]), std::fabs(m.hi[k]));
     const auto launch = [&](const float* p, const float* t, double* out, cudaStream_t s) {
+        // (after every allocation of the call: one could take the copy back)
+        const float4* const groups = symmetric ? add_s_groups(c, mi->second, s) : nullptr;
         return groups ? perch::launch_add_nn(groups, m.n_verts, size, p, t, n, out, s)
                       : perch::launch_add_s(m.verts, m.n_verts, p, t, n, symmetric ? 1 : 0, out, s);
     };

@@ -1,5 +1,6 @@
 """The sorted copy of a mesh's vertices that ADD-S reads: made by the first call that
-uses it and charged to the budget then; a captured call does without it."""
+uses it, charged to the budget then, and given back when the budget needs its room; a
+captured call does without it."""
 import numpy as np
 import pytest
 
@@ -66,3 +67,38 @@ def test_captured_calls(P):
             np.testing.assert_allclose(got, P.perch_add_s(ctx.ctx, mid, est, true, True), rtol=1e-13)
             out.zero_()
         del graph
+
+
+def test_given_back_when_the_budget_needs_its_room(P):
+    """The smallest budget that a program manages with when it asks for ADD is enough
+    when it asks for ADD-S."""
+    mesh = scenes.ellipsoid_mesh(0.04, 0.03, 0.05, 21, 20)      # 8 KB of groups
+    est, true = pairs(5)
+    sc = scenes.tabletop_3obj(grid_half=0)
+
+    def program(budget, symmetric):
+        with P.Context(0, hbm_budget_bytes=budget) as ctx:
+            mid = ctx.load_mesh(mesh)
+            first = P.perch_add_s(ctx.ctx, mid, est, true, symmetric)
+            ctx.set_observation(sc)
+            again = P.perch_add_s(ctx.ctx, mid, est, true, symmetric)
+            assert ctx.hbm_used <= budget
+            return first, again
+
+    def fits(budget, symmetric):
+        try:
+            program(budget, symmetric)
+            return True
+        except P.PerchError as e:
+            assert e.status == -3
+            return False
+
+    lo, hi = 1 << 20, 64 << 20
+    assert fits(hi, False)
+    while hi - lo > 1 << 10:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid, False) else (mid, hi)
+    assert fits(hi, True)
+    want = program(64 << 20, True)[0]
+    for got in program(hi, True):
+        np.testing.assert_allclose(got, want, rtol=1e-13)
