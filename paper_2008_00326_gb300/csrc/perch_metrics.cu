@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kAddThreads) k_add_s(const float4* verts, int 
 constexpr int kNnThreads = 128;
 constexpr int kNnWarps = kNnThreads / 32;
 constexpr int kNnCluster = 8;        // blocks per pose pair when there are few pairs
+constexpr int kNnSums = kNnCluster * kNnWarps;   // partial sums of a pair, however many blocks it has
 constexpr int kNnGroups = 1024;      // groups under B held in shared memory
 constexpr float kAddSlack = 1e-5f;
 
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(kNnThreads) k_add_nn(const float4* verts, cons
     __shared__ float4 near_group[kNnGroups];
     __shared__ float4 staged[kNnWarps][32];
     __shared__ float sA[12], sB[12];
-    __shared__ double sum[kNnWarps];
+    __shared__ double sum[kNnSums];
     const cg::cluster_group cluster = cg::this_cluster();
     const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -151,79 +152,83 @@ __global__ void __launch_bounds__(kNnThreads) k_add_nn(const float4* verts, cons
         if (ng <= kNnGroups)
             for (int g = threadIdx.x; g < ng; g += kNnThreads) near_group[g] = sphere_b(g);
         __syncthreads();
-        double acc = 0.0;
-        for (int i = part * kNnWarps + warp; i < ng; i += parts * kNnWarps) {
-            const int vi = 32 * i + lane;
-            const float3 x = xform(sA, __ldg(&verts[vi]));
-            const float4 ci = __ldg(&spheres[i]);
-            const float3 c = xform(sA, ci);
-            const float reach = ci.w * fa + slack;
-            // distance from the warp's centre to group g's sphere
-            const auto gap = [&](int g) {
-                const float4 s = ng <= kNnGroups ? near_group[g] : sphere_b(g);
-                const float dx = c.x - s.x, dy = c.y - s.y, dz = c.z - s.z;
-                return sqrtf(dx * dx + dy * dy + dz * dz) - s.w;
-            };
-            float best = 3.0e38f;
-            const auto visit = [&](int g) {
-                const float3 y = xform(sB, __ldg(&verts[32 * g + lane]));
-                staged[warp][lane] = 32 * g + lane < nv ? make_float4(y.x, y.y, y.z, 0.0f)
-                                                        : make_float4(1.0e30f, 1.0e30f, 1.0e30f, 0.0f);
-                __syncwarp();
+        // group i goes to partial sum i % kNnSums and a warp adds up whole partial
+        // sums, so that a pair's mean has one summation order and does not depend on
+        // the number of pairs that share the call
+        const int n_sums = min(kNnSums, ng);
+        for (int slot = part * kNnWarps + warp; slot < n_sums; slot += parts * kNnWarps) {
+            double acc = 0.0;
+            for (int i = slot; i < ng; i += kNnSums) {
+                const int vi = 32 * i + lane;
+                const float3 x = xform(sA, __ldg(&verts[vi]));
+                const float4 ci = __ldg(&spheres[i]);
+                const float3 c = xform(sA, ci);
+                const float reach = ci.w * fa + slack;
+                // distance from the warp's centre to group g's sphere
+                const auto gap = [&](int g) {
+                    const float4 s = ng <= kNnGroups ? near_group[g] : sphere_b(g);
+                    const float dx = c.x - s.x, dy = c.y - s.y, dz = c.z - s.z;
+                    return sqrtf(dx * dx + dy * dy + dz * dz) - s.w;
+                };
+                float best = 3.0e38f;
+                const auto visit = [&](int g) {
+                    const float3 y = xform(sB, __ldg(&verts[32 * g + lane]));
+                    staged[warp][lane] = 32 * g + lane < nv ? make_float4(y.x, y.y, y.z, 0.0f)
+                                                            : make_float4(1.0e30f, 1.0e30f, 1.0e30f, 0.0f);
+                    __syncwarp();
 #pragma unroll 8
-                for (int k = 0; k < 32; ++k) {
-                    const float4 p = staged[warp][k];
-                    const float dx = x.x - p.x, dy = x.y - p.y, dz = x.z - p.z;
-                    best = fminf(best, dx * dx + dy * dy + dz * dz);
-                }
-                __syncwarp();
-            };
-            // the group whose sphere is nearest first (any group if none compares)
-            float low = 3.0e38f;
-            int first = 0;
-            for (int g = lane; g < ng; g += 32) {
-                const float d = gap(g);
-                if (d < low) { low = d; first = g; }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const float d = __shfl_xor_sync(0xffffffffu, low, o);
-                const int g = __shfl_xor_sync(0xffffffffu, first, o);
-                if (d < low || (d == low && g < first)) { low = d; first = g; }
-            }
-            visit(first);
-            for (int g0 = 0; g0 < ng; g0 += 32) {
-                // of these 32 groups the nearest first, as long as it is within what the lanes'
-                // worst nearest distance reaches (distances are non-negative: their bits order
-                // like the values; a gap below zero counts as zero, one that does not compare too)
-                const int g = g0 + lane;
-                unsigned ahead = 0xFFFFFFFFu;
-                if (g < ng && g != first) {
+                    for (int k = 0; k < 32; ++k) {
+                        const float4 p = staged[warp][k];
+                        const float dx = x.x - p.x, dy = x.y - p.y, dz = x.z - p.z;
+                        best = fminf(best, dx * dx + dy * dy + dz * dz);
+                    }
+                    __syncwarp();
+                };
+                // the group whose sphere is nearest first (any group if none compares)
+                float low = 3.0e38f;
+                int first = 0;
+                for (int g = lane; g < ng; g += 32) {
                     const float d = gap(g);
-                    ahead = d > 0.0f ? __float_as_uint(d) : 0u;
+                    if (d < low) { low = d; first = g; }
                 }
-                for (;;) {
-                    const unsigned next = __reduce_min_sync(0xffffffffu, ahead);
-                    const float worst = __uint_as_float(__reduce_max_sync(0xffffffffu, vi < nv ? __float_as_uint(best) : 0u));
-                    const float limit = sqrtf(worst) * 1.00001f + reach;
-                    if (next == 0xFFFFFFFFu || __uint_as_float(next) > limit) break;
-                    const unsigned at = __ballot_sync(0xffffffffu, ahead == next);
-                    const int k = __ffs(at) - 1;
-                    if (lane == k) ahead = 0xFFFFFFFFu;
-                    visit(g0 + k);
+                for (int o = 16; o > 0; o >>= 1) {
+                    const float d = __shfl_xor_sync(0xffffffffu, low, o);
+                    const int g = __shfl_xor_sync(0xffffffffu, first, o);
+                    if (d < low || (d == low && g < first)) { low = d; first = g; }
                 }
+                visit(first);
+                for (int g0 = 0; g0 < ng; g0 += 32) {
+                    // of these 32 groups the nearest first, as long as it is within what the lanes'
+                    // worst nearest distance reaches (distances are non-negative: their bits order
+                    // like the values; a gap below zero counts as zero, one that does not compare too)
+                    const int g = g0 + lane;
+                    unsigned ahead = 0xFFFFFFFFu;
+                    if (g < ng && g != first) {
+                        const float d = gap(g);
+                        ahead = d > 0.0f ? __float_as_uint(d) : 0u;
+                    }
+                    for (;;) {
+                        const unsigned next = __reduce_min_sync(0xffffffffu, ahead);
+                        const float worst =
+                            __uint_as_float(__reduce_max_sync(0xffffffffu, vi < nv ? __float_as_uint(best) : 0u));
+                        const float limit = sqrtf(worst) * 1.00001f + reach;
+                        if (next == 0xFFFFFFFFu || __uint_as_float(next) > limit) break;
+                        const unsigned at = __ballot_sync(0xffffffffu, ahead == next);
+                        const int k = __ffs(at) - 1;
+                        if (lane == k) ahead = 0xFFFFFFFFu;
+                        visit(g0 + k);
+                    }
+                }
+                if (vi < nv) acc += sqrt((double)best);
             }
-            if (vi < nv) acc += sqrt((double)best);
-        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) sum[warp] = acc;
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) sum[slot] = acc;
+        }
         cluster.sync();
         if (part == 0 && threadIdx.x == 0) {
             double total = 0.0;
-            for (int b = 0; b < parts; ++b) {
-                const double* const other = cluster.map_shared_rank(sum, b);
-                for (int w = 0; w < kNnWarps; ++w) total += other[w];
-            }
+            for (int k = 0; k < n_sums; ++k) total += cluster.map_shared_rank(sum, k / kNnWarps % parts)[k];
             out[q] = total / (double)nv;
         }
         cluster.sync();              // the sums have been read, and with them the pose arrays
