@@ -493,8 +493,10 @@ perch_status build_hash(perch_ctx* c, SceneRec& s, const uint8_t* d_rgb, long lo
     void *slot = nullptr, *keys = nullptr, *count = nullptr, *cursor = nullptr, *start = nullptr, *nvalid = nullptr,
          *big = nullptr, *occ = nullptr;
     auto cleanup = [&](perch_status r) {
-        dfree(c, slot); dfree(c, keys); dfree(c, count); dfree(c, cursor);
-        dfree(c, start); dfree(c, nvalid); dfree(c, big); dfree(c, occ);
+        for (void** p : {&slot, &keys, &count, &cursor, &start, &nvalid, &big, &occ}) {
+            dfree(c, *p);
+            *p = nullptr;
+        }
         return r;
     };
     if ((st = dalloc(c, std::max<long long>(1, n_valid) * sizeof(float4), &s.pts)) ||
@@ -536,7 +538,10 @@ perch_status build_hash(perch_ctx* c, SceneRec& s, const uint8_t* d_rgb, long lo
     if ((st = check_device_error(c)) != PERCH_OK) return cleanup(st);
     d.table = (const uint4*)s.table;
     d.table_mask = cap_small - 1;
-    if (n_valid == 0 || cells > (1ll << 27)) return cleanup(PERCH_OK);
+    // the bitmaps take the scratch's room in a budget, and the colours' if need be
+    cleanup(PERCH_OK);
+    c->building = false;
+    if (n_valid == 0 || cells > (1ll << 27)) return PERCH_OK;
     const size_t bytes = (size_t)((cells + 31) / 32) * 4;
     if ((st = dalloc(c, bytes, &s.near)) || (st = dalloc(c, bytes, &occ))) return cleanup(st);
     e = cudaMemsetAsync(s.near, 0, bytes, c->stream);
