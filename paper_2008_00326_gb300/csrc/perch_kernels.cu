@@ -638,13 +638,15 @@ __device__ __forceinline__ bool load_triangle(const C& sc, const float4* verts, 
         float Z = __fadd_rn(__fadd_rn(__fadd_rn(__fmul_rn(P[8], v.x), __fmul_rn(P[9], v.y)),
                                       __fmul_rn(P[10], v.z)), P[11]);
         if (!(Z >= sc.z_near)) return false;
-        float px = __fadd_rn(__fmul_rn(sc.fx, __fdiv_rn(X, Z)), sc.cx);
-        float py = __fadd_rn(__fmul_rn(sc.fy, __fdiv_rn(Y, Z)), sc.cy);
+        const float iz = __frcp_rn(Z);     // = fl(1 / Z), as the division would give
+        const bool fits = fminf(fabsf(X), fminf(fabsf(Y), Z)) > kDivLo && fmaxf(fabsf(X), fmaxf(fabsf(Y), Z)) < kDivHi;
+        float px = __fadd_rn(__fmul_rn(sc.fx, fits ? div_by(X, Z, iz) : div_any(X, Z)), sc.cx);
+        float py = __fadd_rn(__fmul_rn(sc.fy, fits ? div_by(Y, Z, iz) : div_any(Y, Z)), sc.cy);
         float sx = __fmul_rn(px, 16.0f), sy = __fmul_rn(py, 16.0f);
         if (!(sx >= gx0) || !(sx < gx1) || !(sy >= gy0) || !(sy < gy1)) return false;
         o.x[k] = __float2int_rn(sx);
         o.y[k] = __float2int_rn(sy);
-        o.iz[k] = __frcp_rn(Z);        // = fl(1 / Z), as the division would give
+        o.iz[k] = iz;
         o.vid[k] = vids[k];
     }
     return true;
@@ -1280,7 +1282,7 @@ extern __shared__ __align__(16) unsigned char g_smem[];
 // every access is a shared-memory one.
 struct RasterArgs {
     const int4* tris;
-    const unsigned long long* vc; // vertex cache, or nullptr: vertices transformed again (cam)
+    const unsigned long long* vc; // vertex cache (raster_whole: nullptr)
     const int* list;              // the tile's bin, or nullptr: triangles 0 .. n - 1
     int n;
     int tu0, tv0, tu1, tv1, tw;   // tile [tu0,tu1) x [tv0,tv1), row pitch tw
@@ -1288,26 +1290,18 @@ struct RasterArgs {
     int* err;
 };
 
-struct RasterCamera {             // without the vertex cache
-    const float4* verts;
-    const float* P;
-    int W, H;
-    float fx, fy, cx, cy, z_near;
-};
-
 // Depth and z-buffer update of the n <= 32 oldest samples of the ring at `at`:
 // the triangle is read again (its weights and 1/Z in the orientation's order),
 // z = A / ((w0/Z0 + w1/Z1) + w2/Z2) with one division, d = rint(10000 z).
-template <bool K32, bool VC>
-__device__ __forceinline__ void depth_flush(const RasterArgs& a, const RasterCamera& cam, int at, int n, int lane)
+template <bool K32>
+__device__ __forceinline__ void depth_flush(const RasterArgs& a, int at, int n, int lane)
 {
     __syncwarp();
     if (lane < n) {
         const DepthItem e = reinterpret_cast<const DepthItem*>(g_smem + a.ring)[(at + lane) & (kRing - 1)];
         const int4 tv = __ldg(&a.tris[e.tri]);
         TriSetup o;
-        if (VC) load_cached(a.vc, tv, o);
-        else load_triangle(cam, cam.verts, cam.P, tv, o);
+        load_cached(a.vc, tv, o);
         const int A = edge_fn(o.x[0], o.y[0], o.x[1], o.y[1], o.x[2], o.y[2]);
         const int idx = (int)(e.idx & 0xFFFFu);
         const int w0 = e.t0 + (int)((e.idx >> 16) & 1u), wa = e.t1 + (int)((e.idx >> 17) & 1u);
@@ -1347,8 +1341,8 @@ __device__ __forceinline__ void depth_flush(const RasterArgs& a, const RasterCam
 // instructions, against 202k and 159k without the triangle ring.  With it, three
 // 640x480 objects x 29,584 poses 42.0 -> 36.2 ms, five 6-DoF objects of 30,000
 // triangles x 4,096 poses 1.41 times the former rate.
-template <int NT, bool K32, bool VC>
-__device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera cam)
+template <int NT, bool K32>
+__device__ __noinline__ void raster_tile(const RasterArgs a)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -1356,24 +1350,21 @@ __device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera 
     TriStage* const TS = reinterpret_cast<TriStage*>(g_smem + a.scratch + kRing * sizeof(uint4));
     DepthItem* const DQ = reinterpret_cast<DepthItem*>(g_smem + a.ring);
     int head = 0, count = 0, dhead = 0, dcount = 0;     // the rings of triangles and samples
-    // with the vertex cache, pixels are biased like its coordinates
-    constexpr int kPix = VC ? kSnapBias / 16 : 0;
+    constexpr int kPix = kSnapBias / 16;                // pixels are biased like the cached coordinates
     const uint32_t tlo = (uint32_t)(a.tu0 + kPix) | ((uint32_t)(a.tv0 + kPix) << 16);
     const uint32_t thi = (uint32_t)(a.tu1 - 1 + kPix) | ((uint32_t)(a.tv1 - 1 + kPix) << 16);
     // vertex ids are loaded two iterations ahead, the vertices' snapped positions
     // (the low halves of their records) one
     int base = warp * 32, t_next = base + lane;
     uint4 e_next = make_uint4(0u, 0u, 0u, 0u);          // positions and id of the next triangle
-    int4 tv_next = make_int4(0, 0, 0, 0);               // vertex ids of the one after it (VC), else of the next
+    int4 tv_next = make_int4(0, 0, 0, 0);               // vertex ids of the one after it
     if (base + lane < a.n) {
         if (a.list) t_next = a.list[t_next];
         e_next.w = (unsigned)t_next;
         tv_next = __ldg(&a.tris[t_next]);
-        if (VC) {
-            e_next.x = (uint32_t)a.vc[tv_next.x]; e_next.y = (uint32_t)a.vc[tv_next.y]; e_next.z = (uint32_t)a.vc[tv_next.z];
-        }
+        e_next.x = (uint32_t)a.vc[tv_next.x]; e_next.y = (uint32_t)a.vc[tv_next.y]; e_next.z = (uint32_t)a.vc[tv_next.z];
     }
-    if (VC && base + lane + NT < a.n) {
+    if (base + lane + NT < a.n) {
         t_next = a.list ? a.list[base + lane + NT] : base + lane + NT;
         tv_next = __ldg(&a.tris[t_next]);
     }
@@ -1382,35 +1373,20 @@ __device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera 
             const int i = base + lane;
             const int4 tv = tv_next;
             uint4 e = e_next;
-            if (VC) {
-                if (i + NT < a.n) {
-                    e_next = make_uint4((uint32_t)a.vc[tv.x], (uint32_t)a.vc[tv.y], (uint32_t)a.vc[tv.z], (unsigned)t_next);
-                    if (i + 2 * NT < a.n) {
-                        t_next = a.list ? a.list[i + 2 * NT] : i + 2 * NT;
-                        tv_next = __ldg(&a.tris[t_next]);
-                    }
+            if (i + NT < a.n) {
+                e_next = make_uint4((uint32_t)a.vc[tv.x], (uint32_t)a.vc[tv.y], (uint32_t)a.vc[tv.z], (unsigned)t_next);
+                if (i + 2 * NT < a.n) {
+                    t_next = a.list ? a.list[i + 2 * NT] : i + 2 * NT;
+                    tv_next = __ldg(&a.tris[t_next]);
                 }
-            } else if (i + NT < a.n) {
-                t_next = a.list ? a.list[i + NT] : i + NT;
-                tv_next = __ldg(&a.tris[t_next]);
-                e_next.w = (unsigned)t_next;
             }
             base += NT;
             bool some = false;
             if (i < a.n) {
-                if (VC) {
-                    const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
-                    const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
-                    const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
-                    some = __vmaxu2(pl, ph) == ph && (hi & 0xFFFFu) != 0xFFFFu;
-                } else {
-                    TriSetup o;
-                    some = load_triangle(cam, cam.verts, cam.P, tv, o) &&
-                           max(ceil16(min(o.x[0], min(o.x[1], o.x[2]))), a.tu0) <=
-                               min(floor16(max(o.x[0], max(o.x[1], o.x[2]))), a.tu1 - 1) &&
-                           max(ceil16(min(o.y[0], min(o.y[1], o.y[2]))), a.tv0) <=
-                               min(floor16(max(o.y[0], max(o.y[1], o.y[2]))), a.tv1 - 1);
-                }
+                const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
+                const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
+                const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
+                some = __vmaxu2(pl, ph) == ph && (hi & 0xFFFFu) != 0xFFFFu;
             }
             const unsigned bal = __ballot_sync(0xffffffffu, some);
             if (some) TR[(head + count + __popc(bal & lt)) & (kRing - 1)] = e;
@@ -1430,25 +1406,13 @@ __device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera 
             tri = (int)e.w;
             head = (head + 32) & (kRing - 1);
             count = max(0, count - 32);
-            int x[3], y[3], u0, v0, bh;
-            if (VC) {
-                const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
-                const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
-                const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
-                u0 = (int)(pl & 0xFFFFu); v0 = (int)(pl >> 16);
-                bw = (int)(ph & 0xFFFFu) - u0 + 1; bh = (int)(ph >> 16) - v0 + 1;
-                x[0] = (int)(e.x & 0xFFFFu); x[1] = (int)(e.y & 0xFFFFu); x[2] = (int)(e.z & 0xFFFFu);
-                y[0] = (int)(e.x >> 16); y[1] = (int)(e.y >> 16); y[2] = (int)(e.z >> 16);
-            } else {
-                TriSetup o;
-                for (int k = 0; k < 3; ++k) o.x[k] = o.y[k] = 0;
-                if (have) load_triangle(cam, cam.verts, cam.P, __ldg(&a.tris[tri]), o);
-                for (int k = 0; k < 3; ++k) { x[k] = o.x[k]; y[k] = o.y[k]; }
-                u0 = max(ceil16(min(x[0], min(x[1], x[2]))), a.tu0);
-                v0 = max(ceil16(min(y[0], min(y[1], y[2]))), a.tv0);
-                bw = min(floor16(max(x[0], max(x[1], x[2]))), a.tu1 - 1) - u0 + 1;
-                bh = min(floor16(max(y[0], max(y[1], y[2]))), a.tv1 - 1) - v0 + 1;
-            }
+            const uint32_t lo = __vimin3_u16x2(e.x, e.y, e.z), hi = __vimax3_u16x2(e.x, e.y, e.z);
+            const uint32_t pl = __vmaxu2(((lo + 0x000F000Fu) >> 4) & 0x0FFF0FFFu, tlo);
+            const uint32_t ph = __vminu2((hi >> 4) & 0x0FFF0FFFu, thi);
+            const int u0 = (int)(pl & 0xFFFFu), v0 = (int)(pl >> 16), bh = (int)(ph >> 16) - v0 + 1;
+            bw = (int)(ph & 0xFFFFu) - u0 + 1;
+            const int x[3] = {(int)(e.x & 0xFFFFu), (int)(e.y & 0xFFFFu), (int)(e.z & 0xFFFFu)};
+            const int y[3] = {(int)(e.x >> 16), (int)(e.y >> 16), (int)(e.z >> 16)};
             // edge i runs from vertex i + 1 to vertex i + 2 (mod 3), all reversed when
             // the area is negative (two-sided rendering)
             int A = edge_fn(x[0], y[0], x[1], y[1], x[2], y[2]);
@@ -1507,7 +1471,7 @@ __device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera 
                 if (wrap) du = bw;
                 if (dcount >= 32 || last) {
                     const int n = min(dcount, 32);
-                    depth_flush<K32, VC>(a, cam, dhead, n, lane);
+                    depth_flush<K32>(a, dhead, n, lane);
                     dhead = (dhead + n) & (kRing - 1);
                     dcount -= n;
                 }
@@ -1557,7 +1521,158 @@ __device__ __noinline__ void raster_tile(const RasterArgs a, const RasterCamera 
     }
 }
 
-// raster_tile of mesh m (or of its triangles list[0 .. n_list)) at pose P.
+// ---- rasteriser without the vertex cache (images over 1023 pixels, or a block that
+// found no cache slot)
+
+struct RasterCamera {             // without the vertex cache
+    const float4* verts;
+    const float* P;
+    int W, H;
+    float fx, fy, cx, cy, z_near;
+};
+
+// A triangle staged with all that its samples need, since its vertices would have to
+// be transformed again (64 bytes, 4 x 16-byte moves): TriStage's fields, and the
+// doubled area and the 1/Z of its vertices in the orientation's order.
+struct __align__(16) TriWhole {
+    int a0, a1, b0, b1;
+    int t0, t1, K, A;
+    float iz0, iz1, iz2;
+    int tri;
+    unsigned idx;                 // z-buffer index of the first sample | tie biases of edges 0 and 1 in bits 16 and 17
+    int bw;
+    float rbw;
+    int first;
+};
+static_assert(32 * sizeof(TriWhole) <= kWarpScratch, "a warp's triangles fit its scratch");
+
+// Coverage, depth and z-buffer update of one sample of a staged triangle: x0 and x1 are
+// edges 0 and 1 there less their tie bias, idx its place in the tile of cap words.
+template <bool K32>
+__device__ __forceinline__ void whole_sample(const TriWhole& s, int x0, int x1, int idx, int cap, int* err)
+{
+    if ((x0 | x1 | (int)((unsigned)s.K - (unsigned)x0 - (unsigned)x1)) < 0) return;
+    if (!PERCH_CHECKED((unsigned)idx < (unsigned)cap, err)) return;
+    uint32_t* const zbuf = reinterpret_cast<uint32_t*>(g_smem);
+    // Early out for a sample that cannot beat the depth already stored here: its depth
+    // is at least 1e4 / max(1/Z) less a few 2^-24 relative, so if max(1/Z) (d_here + 2)
+    // < 9999 its depth is at least d_here + 2 and its key is larger.  The stored key
+    // only decreases, so reading it while other samples update it can only make this
+    // test skip less.
+    unsigned dh;
+    if (K32) {
+        const uint32_t w = zbuf[idx];
+        dh = w == 0xFFFFFFFFu ? 0xFFFFFFFFu : (w >> 16);
+    } else {
+        const unsigned long long w = reinterpret_cast<const unsigned long long*>(zbuf)[idx];
+        dh = w == kEmptyKey ? 0xFFFFFFFFu : (unsigned)(w >> 32);
+    }
+    const float izmax = fmaxf(s.iz0, fmaxf(s.iz1, s.iz2));
+    if (dh < 0xFFFFFFF0u && __fmul_rn(izmax, __uint2float_rn(dh + 2u)) < 9999.0f) return;
+    const int w0 = x0 + (int)((s.idx >> 16) & 1u), w1 = x1 + (int)((s.idx >> 17) & 1u);
+    const int w2 = (int)((unsigned)s.A - (unsigned)w0 - (unsigned)w1);
+    const float num = __fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(w0), s.iz0), __fmul_rn(__int2float_rn(w1), s.iz1)),
+                                __fmul_rn(__int2float_rn(w2), s.iz2));
+    const float dz = __fmul_rn(__fdiv_rn(__int2float_rn(s.A), num), 10000.0f);
+    if (dz < 4294967296.0f) {                           // (as in depth_flush)
+        const unsigned d = __float2uint_rn(dz);
+        if (d >= 1u) zmin<K32>(zbuf, idx, d, s.tri, err);
+    }
+}
+
+// The tile's triangles, 32 at a time, one per lane: transformed and set up once.
+// Boxes of one sample are tested in their lanes; the others are staged and their
+// samples spread evenly over the lanes.  Without the cache every z-buffer tile
+// transforms the mesh again; reading a triangle's vertices for its set-up and for each
+// covered sample too, as raster_tile does, took 1.1 to 1.8 times as long (700 poses at
+// 1,200x380, 20,000 triangles, stride 2: 2.47 against 1.35 ms).
+template <int NT, bool K32>
+__device__ __noinline__ void raster_whole(const RasterArgs a, const RasterCamera cam)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    TriWhole* const TS = reinterpret_cast<TriWhole*>(g_smem + a.scratch);
+    const int cap = a.tw * (a.tv1 - a.tv0);
+    int t_next = 0;                                     // the lane's next triangle, loaded one iteration ahead
+    int4 tv_next = make_int4(0, 0, 0, 0);
+    if (warp * 32 + lane < a.n) {
+        t_next = a.list ? a.list[warp * 32 + lane] : warp * 32 + lane;
+        tv_next = __ldg(&a.tris[t_next]);
+    }
+    for (int base = warp * 32; base < a.n; base += NT) {
+        const int i = base + lane, t = t_next;
+        const int4 tv = tv_next;
+        if (i + NT < a.n) {
+            t_next = a.list ? a.list[i + NT] : i + NT;
+            tv_next = __ldg(&a.tris[t_next]);
+        }
+        int area = 0;
+        TriWhole s = {};
+        TriSetup o;
+        // the box first: many triangles hold no sample of the tile
+        if (i < a.n && load_triangle(cam, cam.verts, cam.P, tv, o)) {
+            const int u0 = max(ceil16(min(o.x[0], min(o.x[1], o.x[2]))), a.tu0);
+            const int u1 = min(floor16(max(o.x[0], max(o.x[1], o.x[2]))), a.tu1 - 1);
+            const int v0 = max(ceil16(min(o.y[0], min(o.y[1], o.y[2]))), a.tv0);
+            const int v1 = min(floor16(max(o.y[0], max(o.y[1], o.y[2]))), a.tv1 - 1);
+            if (u0 <= u1 && v0 <= v1 && orient_triangle(o)) {
+                const int dx0 = o.x[2] - o.x[1], dy0 = o.y[2] - o.y[1], dx1 = o.x[0] - o.x[2], dy1 = o.y[0] - o.y[2];
+                const int n0 = owns(dx0, dy0) ? 0 : 1, n1 = owns(dx1, dy1) ? 0 : 1;
+                s.a0 = -16 * dy0; s.a1 = -16 * dy1;
+                s.b0 = 16 * dx0; s.b1 = 16 * dx1;
+                s.t0 = (int)((unsigned)dx0 * (unsigned)(16 * v0 - o.y[1]) - (unsigned)dy0 * (unsigned)(16 * u0 - o.x[1]) -
+                             (unsigned)n0);
+                s.t1 = (int)((unsigned)dx1 * (unsigned)(16 * v0 - o.y[2]) - (unsigned)dy1 * (unsigned)(16 * u0 - o.x[2]) -
+                             (unsigned)n1);
+                s.K = o.A - n0 - n1 - (owns(o.x[1] - o.x[0], o.y[1] - o.y[0]) ? 0 : 1);
+                s.A = o.A;
+                s.iz0 = o.iz[0]; s.iz1 = o.iz[1]; s.iz2 = o.iz[2];
+                s.tri = t;
+                s.idx = (unsigned)((v0 - a.tv0) * a.tw + (u0 - a.tu0)) | (unsigned)((n0 << 16) | (n1 << 17));
+                s.bw = u1 - u0 + 1;
+                s.rbw = __frcp_rn(__int2float_rn(s.bw));
+                area = s.bw * (v1 - v0 + 1);
+            }
+        }
+        if (area == 1) whole_sample<K32>(s, s.t0, s.t1, (int)(s.idx & 0xFFFFu), cap, a.err);
+        const int items = area > 1 ? area : 0;
+        const unsigned some = __ballot_sync(0xffffffffu, items > 0);
+        if (some == 0u) continue;
+        int first = items;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, first, off);
+            if (lane >= off) first += x;
+        }
+        const int total = __shfl_sync(0xffffffffu, first, 31);
+        first -= items;
+        s.first = first;
+        if (items > 0) TS[__popc(some & lt)] = s;
+        __syncwarp();
+        int begun = 0;                                  // staged triangles whose samples began before f0
+        for (int f0 = 0; f0 < total; f0 += 32) {
+            // sample f belongs to the last triangle begun at or before it
+            const unsigned rel = (unsigned)(first - f0);
+            const unsigned starts = __reduce_or_sync(0xffffffffu, items > 0 && rel < 32u ? 1u << rel : 0u);
+            begun += __popc(starts & (lt | (1u << lane)));
+            if (f0 + lane < total) {
+                const TriWhole e = TS[begun - 1];
+                const int local = f0 + lane - e.first;
+                int v = __float2int_rz(__fmul_rn(__int2float_rn(local), e.rbw));
+                const int r = local - v * e.bw;
+                v += (r >= e.bw) - (r < 0);
+                const int u = local - v * e.bw;
+                whole_sample<K32>(e, (int)((unsigned)e.t0 + (unsigned)e.b0 * (unsigned)v + (unsigned)e.a0 * (unsigned)u),
+                                  (int)((unsigned)e.t1 + (unsigned)e.b1 * (unsigned)v + (unsigned)e.a1 * (unsigned)u),
+                                  (int)(e.idx & 0xFFFFu) + v * a.tw + u, cap, a.err);
+            }
+            begun = __shfl_sync(0xffffffffu, begun, 31);
+        }
+        __syncwarp();
+    }
+}
+
+// The tile's render of mesh m (or of its triangles list[0 .. n_list)) at pose P.
 // probe_off and ring_off: byte offsets of the block's per-warp scratch and of its
 // warps' depth rings in shared memory.
 template <int NT, bool K32, bool VC>
@@ -1570,9 +1685,10 @@ __device__ __forceinline__ void raster(const DevScene& sc, const DevMesh& m, con
     const RasterArgs a = {m.tris, vc, list, list ? n_list : m.n_tris, tu0, tv0, tu1, tv1, tw,
                           probe_off + warp * (unsigned)kWarpScratch,
                           ring_off + warp * (unsigned)(kRing * sizeof(DepthItem)), err};
-    RasterCamera cam = {};
-    if (!VC) cam = {m.verts, P, sc.W, sc.H, sc.fx, sc.fy, sc.cx, sc.cy, sc.z_near};
-    raster_tile<NT, K32, VC>(a, cam);
+    if (VC)
+        raster_tile<NT, K32>(a);
+    else
+        raster_whole<NT, K32>(a, RasterCamera{m.verts, P, sc.W, sc.H, sc.fx, sc.fy, sc.cx, sc.cy, sc.z_near});
 }
 
 // Tile bins of one hypothesis: the pixel box rbox is rasterised in tiles of tw
