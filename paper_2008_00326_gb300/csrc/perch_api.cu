@@ -782,6 +782,7 @@ perch_status perch_load_mesh(perch_ctx* c, const float* verts_xyz, const uint8_t
         }
         t4[4 * i + 3] = 0;
     }
+    const bool stout = perch::stout_triangles(v4.data(), t4.data(), n_tris);
     DeviceGuard g(c->device);
     std::lock_guard<std::mutex> lk(c->mu);
     Range r("perch: mesh upload");
@@ -804,6 +805,7 @@ perch_status perch_load_mesh(perch_ctx* c, const float* verts_xyz, const uint8_t
     rec.dm.tris = (const int4*)rec.tris;
     rec.dm.n_verts = n_verts;
     rec.dm.n_tris = n_tris;
+    rec.dm.stout = stout;
     rec.dm.vol_r = vol_radius_m;
     rec.dm.vol_h = vol_height_m;
     for (int k = 0; k < 3; ++k) {

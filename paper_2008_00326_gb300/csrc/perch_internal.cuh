@@ -2,6 +2,8 @@
 // (perch_kernels.cu) of libperch.  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -45,9 +47,33 @@ struct DevMesh {
     const float4* verts;      // (x, y, z, rgb packed in the low 24 bits of w's bit pattern)
     const int4* tris;         // (a, b, c, 0)
     int n_verts, n_tris;
+    int stout;                // its triangles fill their boxes (stout_triangles)
     float vol_r, vol_h;
     float lo[3], hi[3];       // object-frame bounding box of the vertices
 };
+
+// Do the triangles (four words each) of packed vertices fill a good part of their
+// boxes, or are they thin wedges and slivers?  The squared longest edges summed over
+// the areas summed is 2.3 for equilateral ones, 4 for halves of squares, and 9.5 and 11
+// for finely divided cylinders with end caps of 64 and 100 wedges: the line is 8.  Over
+// some 4,096 of them, evenly spaced (0.1 ms).
+inline bool stout_triangles(const float* v4, const int32_t* t4, int n_tris)
+{
+    double edges2 = 0.0, areas = 0.0;
+    for (int i = 0; i < n_tris; i += 1 + n_tris / 4096) {
+        double e[3][3], longest = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            const float *p = v4 + 4 * (size_t)t4[4 * (size_t)i + a], *q = v4 + 4 * (size_t)t4[4 * (size_t)i + (a + 1) % 3];
+            for (int k = 0; k < 3; ++k) e[a][k] = (double)q[k] - p[k];
+            longest = std::max(longest, e[a][0] * e[a][0] + e[a][1] * e[a][1] + e[a][2] * e[a][2]);
+        }
+        const double nx = e[0][1] * e[1][2] - e[0][2] * e[1][1], ny = e[0][2] * e[1][0] - e[0][0] * e[1][2];
+        const double nz = e[0][0] * e[1][1] - e[0][1] * e[1][0];
+        edges2 += longest;
+        areas += 0.5 * std::sqrt(nx * nx + ny * ny + nz * nz);
+    }
+    return edges2 <= 8.0 * areas;
+}
 
 // A state of the Monotone Scene Generation tree (the objects placed so
 // far) as per-pixel images, for scoring the edges that add one more object.

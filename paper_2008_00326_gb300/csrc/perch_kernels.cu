@@ -1521,8 +1521,8 @@ __device__ __noinline__ void raster_tile(const RasterArgs a)
     }
 }
 
-// ---- rasteriser without the vertex cache (images over 1023 pixels, or a block that
-// found no cache slot)
+// ---- rasteriser of staged triangles: large ones, or no vertex cache (images over 1023
+// pixels, or a block that found no cache slot)
 
 struct RasterCamera {             // without the vertex cache
     const float4* verts;
@@ -1530,6 +1530,7 @@ struct RasterCamera {             // without the vertex cache
     int W, H;
     float fx, fy, cx, cy, z_near;
 };
+struct CachedVertices {};         // with it
 
 // A triangle staged with all that its samples need, since its vertices would have to
 // be transformed again (64 bytes, 4 x 16-byte moves): TriStage's fields, and the
@@ -1545,6 +1546,16 @@ struct __align__(16) TriWhole {
     int first;
 };
 static_assert(32 * sizeof(TriWhole) <= kWarpScratch, "a warp's triangles fit its scratch");
+
+// A triangle's snapped positions and 1/Z, from the vertex cache or transformed here.
+__device__ __forceinline__ bool load_whole(const RasterArgs& a, CachedVertices, int4 tv, TriSetup& o)
+{
+    return load_cached(a.vc, tv, o);
+}
+__device__ __forceinline__ bool load_whole(const RasterArgs&, const RasterCamera& c, int4 tv, TriSetup& o)
+{
+    return load_triangle(c, c.verts, c.P, tv, o);
+}
 
 // Coverage, depth and z-buffer update of one sample of a staged triangle: x0 and x1 are
 // edges 0 and 1 there less their tie bias, idx its place in the tile of cap words.
@@ -1580,14 +1591,14 @@ __device__ __forceinline__ void whole_sample(const TriWhole& s, int x0, int x1, 
     }
 }
 
-// The tile's triangles, 32 at a time, one per lane: transformed and set up once.
+// The tile's triangles, 32 at a time, one per lane: loaded and set up once.
 // Boxes of one sample are tested in their lanes; the others are staged and their
 // samples spread evenly over the lanes.  Without the cache every z-buffer tile
 // transforms the mesh again; reading a triangle's vertices for its set-up and for each
 // covered sample too, as raster_tile does, took 1.1 to 1.8 times as long (700 poses at
 // 1,200x380, 20,000 triangles, stride 2: 2.47 against 1.35 ms).
-template <int NT, bool K32>
-__device__ __noinline__ void raster_whole(const RasterArgs a, const RasterCamera cam)
+template <int NT, bool K32, class Camera>
+__device__ __noinline__ void raster_whole(const RasterArgs a, const Camera cam)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -1610,7 +1621,7 @@ __device__ __noinline__ void raster_whole(const RasterArgs a, const RasterCamera
         TriWhole s = {};
         TriSetup o;
         // the box first: many triangles hold no sample of the tile
-        if (i < a.n && load_triangle(cam, cam.verts, cam.P, tv, o)) {
+        if (i < a.n && load_whole(a, cam, tv, o)) {
             const int u0 = max(ceil16(min(o.x[0], min(o.x[1], o.x[2]))), a.tu0);
             const int u1 = min(floor16(max(o.x[0], max(o.x[1], o.x[2]))), a.tu1 - 1);
             const int v0 = max(ceil16(min(o.y[0], min(o.y[1], o.y[2]))), a.tv0);
@@ -1672,23 +1683,38 @@ __device__ __noinline__ void raster_whole(const RasterArgs a, const RasterCamera
     }
 }
 
+// Which rasteriser the render of a mesh with stout triangles takes (DevMesh::stout).
+// raster_tile keeps its lanes full where most triangles hold few samples or their boxes
+// few covered ones; where a triangle holds several, setting it up with its depths at
+// hand beats reading it again for each.  us for 1,452 poses, raster_tile /
+// raster_whole, at 160x120, 320x240 and 640x480 (stride 3, mostly render): boxes of 588
+// triangles 128 / 109, 300 / 243, 1,344 / 1,147 and of 10,800 209 / 238, 386 / 433, 1,390
+// / 1,198; ellipsoids of 1,104 103 / 95, 233 / 189, 730 / 641 and of 18,240 232 / 305,
+// 393 / 472, 1,089 / 1,115.  They meet at about one sample a triangle.  A cylinder of
+// 8,200 with end caps of thin wedges, which fill little of their boxes, is the rings'
+// throughout: 193 / 265, 353 / 599, 2,187 / 4,620.
+__device__ __forceinline__ bool few_large_triangles(const DevMesh& m, int px) { return px >= m.n_tris; }
+
 // The tile's render of mesh m (or of its triangles list[0 .. n_list)) at pose P.
 // probe_off and ring_off: byte offsets of the block's per-warp scratch and of its
-// warps' depth rings in shared memory.
-template <int NT, bool K32, bool VC>
+// warps' depth rings in shared memory.  EITHER: the rasteriser is chosen by the px
+// samples of the hypothesis's whole render, else raster_tile with the vertex cache.
+template <int NT, bool K32, bool VC, bool EITHER = false>
 __device__ __forceinline__ void raster(const DevScene& sc, const DevMesh& m, const float* P,
                                        const unsigned long long* vc, unsigned probe_off, unsigned ring_off, int tu0,
                                        int tv0, int tu1, int tv1, int tw, int* err, const int* list = nullptr,
-                                       int n_list = 0)
+                                       int n_list = 0, int px = 0)
 {
     const unsigned warp = threadIdx.x >> 5;
     const RasterArgs a = {m.tris, vc, list, list ? n_list : m.n_tris, tu0, tv0, tu1, tv1, tw,
                           probe_off + warp * (unsigned)kWarpScratch,
                           ring_off + warp * (unsigned)(kRing * sizeof(DepthItem)), err};
-    if (VC)
-        raster_tile<NT, K32>(a);
-    else
+    if (!VC)
         raster_whole<NT, K32>(a, RasterCamera{m.verts, P, sc.W, sc.H, sc.fx, sc.fy, sc.cx, sc.cy, sc.z_near});
+    else if (EITHER && few_large_triangles(m, px))
+        raster_whole<NT, K32>(a, CachedVertices{});
+    else
+        raster_tile<NT, K32>(a);
 }
 
 // Tile bins of one hypothesis: the pixel box rbox is rasterised in tiles of tw
@@ -1802,6 +1828,16 @@ __device__ __forceinline__ void jo_colour_pass(const Job& J, const float* P, con
 // plain path carries none of the other two's code.
 enum : int { kModePlain = 0, kModeTree = 1, kModeEq3 = 2 };
 
+// Forms of plain scoring, compiled separately too: the rings' rasteriser alone, with
+// tile bins, or the choice between the two rasterisers.  The choice in every kernel cost
+// the renders that never take it 1 to 3 % (three 640x480 objects x 29,584 poses 36.5
+// against 35.9 ms, the tree search 53.4 against 51.6), so it is compiled for meshes that
+// can gain by it: stout triangles, no more of them than the region of interest holds
+// pixels nor than kEitherTris (a render of more samples than that takes three tiles).
+// The other modes search and count more than they render, and take the rings.
+enum : int { kFormRings = 0, kFormBins = 1, kFormEither = 2 };
+constexpr int kEitherTris = 16384;
+
 // Is the observed point p of pixel pix in the admissible set V(O) at pose P
 // (Sec. IV-A J_o; labels Sec. V-C)?  The inscribed cylinder about the
 // object's z-axis (radius^2 rr, height vol_h) in the object frame, R^T (p - t),
@@ -1851,12 +1887,12 @@ __device__ __forceinline__ void jo_count_in(const DevScene& sc, const Job& J, co
 // Rasterise, resolve and radius-search the pixel box rbox in z-buffer tiles.
 // J_r is accumulated when count_jr; marks are set for nearest neighbours that
 // fall in rows [mv0, mv1) of the admissible box vbox.
-template <int NT, bool K32, bool VC, int MODE, bool BINS>
+template <int NT, bool K32, bool VC, int MODE, int FORM>
 __device__ __forceinline__ void score_tiles(const ScoreArgs& a, const Job& J, const float* P, const unsigned long long* vc,
                             const int* rbox, const ScoreSmem& S, const int* vbox, int mv0, int mv1,
                             bool count_jr, int& jr_local, int& n_in, int& n_marked)
 {
-    constexpr bool TREE = MODE == kModeTree, EQ3 = MODE == kModeEq3;
+    constexpr bool TREE = MODE == kModeTree, EQ3 = MODE == kModeEq3, BINS = FORM == kFormBins;
     const DevScene& sc = J.sc;
     const float rr = __fmul_rn(J.m.vol_r, J.m.vol_r);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1897,8 +1933,9 @@ __device__ __forceinline__ void score_tiles(const ScoreArgs& a, const Job& J, co
             // (the depth rings take the place of the kept-point queues, idle meanwhile)
             const bool in_bin = BINS && binned && S.bin_cnt[tile] <= a.bin_cap;
             if (MODE != kModePlain || (rw > 0 && rh > 0))
-                raster<NT, K32, VC>(sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw, a.err,
-                                    in_bin ? bins + tile * a.bin_cap : nullptr, in_bin ? S.bin_cnt[tile] : 0);
+                raster<NT, K32, VC, FORM == kFormEither>(sc, J.m, P, vc, a.probe_off, a.kept_off, tu0, tv0, tu1, tv1, tw,
+                                                         a.err, in_bin ? bins + tile * a.bin_cap : nullptr,
+                                                         in_bin ? S.bin_cnt[tile] : 0, rw * rh);
             __syncthreads();
             if (a.dump) {
                 for (int i = threadIdx.x; i < tpx; i += NT) {
@@ -2060,18 +2097,18 @@ __device__ __forceinline__ void score_tiles(const ScoreArgs& a, const Job& J, co
 // keys (65,536 triangles or more, poses beyond 6.5 m): called, so that the
 // common case has the kernel's registers and instruction cache to itself.
 // Returns (J_r, |I cap V|, marked) of this thread.
-template <int NT, int MODE, bool BINS>
+template <int NT, int MODE, int FORM>
 __device__ __noinline__ int3 score_tiles_rare(const ScoreArgs& a, const float* P, const unsigned long long* vc,
                                               const int* rbox, ScoreSmem S, const int* vbox, int mv0, int mv1,
                                               bool count_jr, int k32)
 {
     int3 r = make_int3(0, 0, 0);
     if (vc)
-        score_tiles<NT, false, true, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+        score_tiles<NT, false, true, MODE, FORM>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
     else if (k32)
-        score_tiles<NT, true, false, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+        score_tiles<NT, true, false, MODE, FORM>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
     else
-        score_tiles<NT, false, false, MODE, BINS>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
+        score_tiles<NT, false, false, MODE, FORM>(a, a.job, P, vc, rbox, S, vbox, mv0, mv1, count_jr, r.x, r.y, r.z);
     return r;
 }
 
@@ -2109,7 +2146,7 @@ __device__ __noinline__ void jo_colour_band(const ScoreArgs& a, const Job& J, co
 }
 
 // Score hypothesis h (one block).  Writes costs[2h] = J_o, costs[2h+1] = J_r.
-template <int NT, int MODE, bool BINS>
+template <int NT, int MODE, int FORM>
 __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const ScoreSmem& S, float* s_pose,
                           int* s_rbox, int* s_vbox, int* s_k32, int (*s_red)[NT / 32],
                           unsigned long long* vc)
@@ -2178,9 +2215,9 @@ __device__ void score_one(const ScoreArgs& a, const Job& J, long long h, const S
         for (int i = threadIdx.x; i < mwords; i += NT) S.marks[i] = mfill;
         __syncthreads();
         if (*s_k32 && use_vc) {
-            score_tiles<NT, true, true, MODE, BINS>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, jr, n_in, n_marked);
+            score_tiles<NT, true, true, MODE, FORM>(a, J, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, jr, n_in, n_marked);
         } else {
-            const int3 r = score_tiles_rare<NT, MODE, BINS>(a, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, *s_k32);
+            const int3 r = score_tiles_rare<NT, MODE, FORM>(a, P, vc, s_rbox, S, s_vbox, mv0, mv1, band == 0, *s_k32);
             jr += r.x;
             n_in += r.y;
             n_marked += r.z;
@@ -2329,7 +2366,7 @@ __device__ int claim_vslot(unsigned* mask, int nslots)
 // 39.9 ms for three 640x480 objects x 29,584 poses).  The Eq. 3 scorer, which
 // holds more, would run from spilled values: 80 registers (2.44 against 2.84 ms
 // for two objects x 2,527 poses at 517x389).
-template <int NT, int MODE, bool BINS>
+template <int NT, int MODE, int FORM>
 __global__ void __launch_bounds__(NT, NT == 512 ? 1 : (MODE == kModeEq3 ? 768 : 1024) / NT) k_score(const __grid_constant__ ScoreArgs a)
 {
     unsigned char* const smem = g_smem;
@@ -2355,7 +2392,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : (MODE == kModeEq3 ? 768 : 
         __syncthreads();
         const long long h = s_h;
         if (h >= a.n) break;
-        score_one<NT, MODE, BINS>(a, a.job, h, S, s_pose, s_rbox, s_vbox, &s_k32, s_red, vc);
+        score_one<NT, MODE, FORM>(a, a.job, h, S, s_pose, s_rbox, s_vbox, &s_k32, s_red, vc);
     }
     // every thread has passed the barrier after its last use of the slot
     if (threadIdx.x == 0 && s_slot >= 0) {
@@ -2390,14 +2427,14 @@ static cudaError_t allow_smem(const void* fn)
     return e;
 }
 
-template <int NT, int MODE, bool BINS>
+template <int NT, int MODE, int FORM>
 static int score_grid_nt(size_t smem)
 {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (allow_smem((const void*)k_score<NT, MODE, BINS>) != cudaSuccess) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_score<NT, MODE, BINS>, NT, smem) != cudaSuccess)
+    if (allow_smem((const void*)k_score<NT, MODE, FORM>) != cudaSuccess) return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_score<NT, MODE, FORM>, NT, smem) != cudaSuccess)
         return -1;
     return max(1, per) * max(1, sms);
 }
@@ -2408,10 +2445,11 @@ static int score_grid_all(size_t smem)
     // the specialisations share one grid and one vertex-cache pool: sized for the
     // one with most resident blocks (of another, the blocks past its own share
     // start as others end and find the counter spent)
-    const int g[4] = {score_grid_nt<NT, kModePlain, false>(smem), score_grid_nt<NT, kModePlain, true>(smem),
-                      score_grid_nt<NT, kModeTree, false>(smem), score_grid_nt<NT, kModeEq3, false>(smem)};
+    const int g[5] = {score_grid_nt<NT, kModePlain, kFormRings>(smem), score_grid_nt<NT, kModePlain, kFormBins>(smem),
+                      score_grid_nt<NT, kModePlain, kFormEither>(smem), score_grid_nt<NT, kModeTree, kFormRings>(smem),
+                      score_grid_nt<NT, kModeEq3, kFormRings>(smem)};
     int most = g[0];
-    for (int k = 1; k < 4; ++k) most = g[k] < 0 || most < 0 ? -1 : max(most, g[k]);
+    for (int k = 1; k < 5; ++k) most = g[k] < 0 || most < 0 ? -1 : max(most, g[k]);
     return most;
 }
 
@@ -2449,10 +2487,13 @@ static ScoreArgs with_layout(ScoreArgs a, int threads)
 template <int NT>
 static const void* score_kernel(const ScoreArgs& a)
 {
-    if (a.job.tree.depth) return (const void*)k_score<NT, kModeTree, false>;
-    if (a.job.sc.jo_mode == 1) return (const void*)k_score<NT, kModeEq3, false>;
-    if (a.bin_cap > 0) return (const void*)k_score<NT, kModePlain, true>;
-    return (const void*)k_score<NT, kModePlain, false>;
+    const Job& J = a.job;
+    if (J.tree.depth) return (const void*)k_score<NT, kModeTree, kFormRings>;
+    if (J.sc.jo_mode == 1) return (const void*)k_score<NT, kModeEq3, kFormRings>;
+    if (a.bin_cap > 0) return (const void*)k_score<NT, kModePlain, kFormBins>;
+    const long long px = (long long)(J.roi[2] - J.roi[0]) * (J.roi[3] - J.roi[1]);
+    if (J.m.stout && J.m.n_tris <= kEitherTris && J.m.n_tris <= px) return (const void*)k_score<NT, kModePlain, kFormEither>;
+    return (const void*)k_score<NT, kModePlain, kFormRings>;
 }
 
 template <int NT>
