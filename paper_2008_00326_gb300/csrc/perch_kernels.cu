@@ -761,7 +761,7 @@ struct MarkBand {
 // within delta that lies in the admissible band: its nearest rendered point
 // is the smallest (d2, rendered pixel), the rendered pixel carried in q.w.
 template <bool MARK>
-__device__ __forceinline__ unsigned long long scan_staged(const DevScene& sc, const float4 q, const float4* stage,
+__device__ __forceinline__ unsigned long long scan_staged(float delta2, const float4 q, const float4* stage,
                                                           int n, int j, int k, const MarkBand& mb,
                                                           unsigned long long local)
 {
@@ -769,7 +769,7 @@ __device__ __forceinline__ unsigned long long scan_staged(const DevScene& sc, co
         const float4 c = stage[i];
         float ex = __fsub_rn(q.x, c.x), ey = __fsub_rn(q.y, c.y), ez = __fsub_rn(q.z, c.z);
         float d2 = __fadd_rn(__fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey)), __fmul_rn(ez, ez));
-        if (d2 <= sc.delta2) {
+        if (d2 <= delta2) {
             unsigned long long key = ((unsigned long long)__float_as_uint(d2) << 32) | __float_as_uint(c.w);
             local = key < local ? key : local;
             if (MARK) {
@@ -819,8 +819,13 @@ __device__ __forceinline__ void stage_chunk(const DevScene& sc, WarpProbe& W, in
 // it into the query's result with one shared-memory atomicMin.
 template <bool MARK>
 __device__ __noinline__ unsigned long long probe_hash(const DevScene& sc, bool valid, float4 query, WarpProbe& W,
-                                                      int lane, const MarkBand& mb)
+                                                      int lane, const MarkBand& band)
 {
+    // copies: the caller's lie in memory that the marks' atomics might change, and were
+    // read again for every candidate (Eq. 3 over 700 poses at 1023x455, 2 mm: 11.2
+    // against 9.4 ms)
+    const MarkBand mb = band;
+    const float delta2 = sc.delta2;
     int cx = 0, cy = 0, cz = 0;
     unsigned long long key = kEmptyKey;
     if (valid) {
@@ -861,7 +866,7 @@ __device__ __noinline__ unsigned long long probe_hash(const DevScene& sc, bool v
             stage_chunk(sc, W, run, c0, T, lane, mb.err);
             __syncwarp();
             const int n = min(64, T - c0);
-            if (active) local = scan_staged<MARK>(sc, q, W.stage, n, lane - qj * k, k, mb, local);
+            if (active) local = scan_staged<MARK>(delta2, q, W.stage, n, lane - qj * k, k, mb, local);
             __syncwarp();
         }
         if (active && local != kEmptyKey) atomicMin(&W.best[ql], local);
