@@ -505,7 +505,11 @@ PERCH_API perch_status perch_tree_search(perch_ctx *ctx, int32_t scene_id, const
  * transforms and distances in binary32, the mean in binary64.  poses and
  * poses_true are n*12 row-major 3x4, add receives n doubles.  cuda_stream
  * NULL: HOST pointers, synchronous; otherwise DEVICE pointers on that stream.
- * ADD-S costs n * V^2 distance evaluations (V vertices).
+ * The first ADD-S call on a mesh sorts its V vertices (host, 1 ms at 10,000) into
+ * a copy charged to the budget and given back when its room is needed; a call
+ * under stream capture, or without room for the copy, costs n * V^2 distance
+ * evaluations, the others a fraction.  The means of the two differ by the order
+ * of their sums alone.
  * perch_add_s_auc (host only): the area under the accuracy curve
  * acc(t) = |{i : add_i < t}| / n for t in [0, max_threshold], divided by
  * max_threshold: the mean of max(0, 1 - add_i / max_threshold). */

@@ -3185,7 +3185,7 @@ cudaError_t launch_proposals(const ProposalArgs& a, cudaStream_t s)
 // equal, 10.3 (13.3).
 constexpr int kBestThreads = 256;
 constexpr int kBestUnroll = 4;
-constexpr int kBestGrid = 4 * 152;       // blocks at most: four per SM
+constexpr int kBestGrid = 608;           // blocks at most, on any device: four per SM of 152
 static_assert(kBestGrid <= kBestMaxBlocks, "a block's result has its place in the scratch");
 
 struct BestKey {
